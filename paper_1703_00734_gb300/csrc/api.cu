@@ -194,10 +194,11 @@ struct bmf_ctx {
     int summary = BMF_SUMMARY_MM, ncomp = 3, max_samples = 0;
     bool independent = false;        // no propagation between stages (cfg.independent)
     // sampled noise precision (cfg.noise): tau per W arena row, the row-side Gram's scaled copy
-    // of W and scaled values (the originals kept), per-row SSE, the batch's subset blocks
+    // of W and scaled values (the originals kept), squared residuals per W work item, the batch's
+    // subset blocks
     int noise = BMF_NOISE_FIXED;
     double noise_a0 = 1.0, noise_b0 = 1.0;
-    double *tau_w = nullptr, *noise_sse = nullptr;
+    double *tau_w = nullptr, *noise_part = nullptr;
     void *Ws = nullptr, *xval_orig = nullptr;
     NoiseBlock *noise_blocks = nullptr;
     std::vector<NoiseBlock> h_noise_blocks;
@@ -1087,10 +1088,10 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             if (c->noise && f == 1) {
                 // the noise precisions given the new X and W, then the scaled copies of the
                 // next sweep's row-side Gram
-                launch_noise_sse(K, rw0, rw1, c->W.ptr, c->W.idx, c->W.val, c->prec, c->X.F, c->W.F,
-                                 c->noise_sse, c->st);
-                launch_noise_tau(c->noise, c->noise_b0, c->noise_blocks, sl1 - sl0, d, c->noise_sse,
-                                 c->tau_w, c->st);
+                launch_noise_sse(K, c->W.items + i0, i1 - i0, c->W.idx, c->W.val, c->prec, c->X.F,
+                                 c->W.F, c->noise_part, c->sms, c->st);
+                launch_noise_tau(c->noise, c->noise_b0, c->noise_blocks, sl1 - sl0, d, c->noise_part,
+                                 c->W.item_ptr, i0, c->tau_w, c->st);
                 noise_scale();
                 c->launches += 3;
             }
@@ -1724,7 +1725,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
         const size_t vb = c->prec == BMF_FP64 ? 8 : 4;
         const int64_t nx = c->X.h_obs[c->P.RX];
         c->tau_w = c->mem.alloc<double>(c->P.RW);
-        c->noise_sse = c->mem.alloc<double>(c->P.RW);
+        c->noise_part = c->mem.alloc<double>(c->W.h_item_ptr[c->P.RW]);
         c->Ws = c->mem.alloc<char>((size_t)c->P.RW * c->ldg * gb);
         c->xval_orig = c->mem.alloc<char>((size_t)nx * vb);
         c->noise_blocks = c->mem.alloc<NoiseBlock>(S);

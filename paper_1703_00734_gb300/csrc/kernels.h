@@ -349,21 +349,22 @@ void launch_gen(const GenParams &p, cudaStream_t st);
 int64_t gen_segments(const std::vector<GenSubset> &subs, int K, double nu0, int noise, double a0,
                      std::vector<GenSeg> &segs);
 
-// Sampled noise precision (Section 2.1).  noise_sse: per W arena row of [r0, r1), the sum of
-// squared residuals over the column's entries (FP64, in order) into sse.  noise_tau: the new
-// precisions from the chi-square variates (column mode: tau = c / (2 b0 + SSE) per row; global
-// mode: per subset block [b0_k, b1_k) one value from the block's summed SSE).  noise_scale:
+// Sampled noise precision (Section 2.1).  noise_sse: per column-side work item, the sum of
+// squared residuals over its entries (FP64) into part.  noise_tau: the new precisions from the
+// chi-square variates and the rows' item sums (item i of the launch at part[i - item0]; column
+// mode: tau = c / (2 b0 + SSE) per row; global mode: per subset one value from its summed SSE).  noise_scale:
 // the scaled copies the row-side Gram takes, Ws[r] = sqrt(tau[r]) W[r] for rows [r0, r1) and
 // val[q] = val_orig[q] sqrt(tau[idx[q]]) for entries [q0, q1).
-void launch_noise_sse(int K, int64_t r0, int64_t r1, const int64_t *ptr, const int32_t *idx,
-                      const void *val, int prec, const double *X, const double *W, double *sse,
-                      cudaStream_t st);
+void launch_noise_sse(int K, const GramItem *items, int64_t n_items, const int32_t *idx,
+                      const void *val, int prec, const double *X, const double *W, double *part,
+                      int sms, cudaStream_t st);
 struct NoiseBlock {
     int64_t r0, r1;      // W arena rows of one subset
     int64_t draw;        // offset of its variates in the sweep's draw buffer
 };
 void launch_noise_tau(int mode, double b0, const NoiseBlock *blocks, int n_blocks,
-                      const double *draws, const double *sse, double *tau, cudaStream_t st);
+                      const double *draws, const double *part, const int64_t *item_ptr,
+                      int64_t item0, double *tau, cudaStream_t st);
 void launch_noise_scale(int K, int prec, int64_t r0, int64_t r1, const double *tau,
                         const double *W, void *Ws, int ldg, int64_t q0, int64_t q1,
                         const int32_t *idx, const void *val_orig, void *val, cudaStream_t st);
