@@ -417,8 +417,8 @@ void bmf_destroy(bmf_ctx *ctx);
  * through its own pool allocator, or a service that must not grow its device footprint after
  * start-up.  This call combines, for R rows, the per-row Gaussians of J submodels by Eq. 14 with
  * the eigenvalue correction of Algorithm 2 (the same operation bmf_posterior_means applies to a
- * context's moment-matched subset posteriors) and allocates nothing: its per-row working
- * matrices live in a static device array of BMF_AGGREGATE_STATIC_MAX_DOUBLES doubles (32 MiB)
+ * context's moment-matched subset posteriors) and allocates nothing: what its
+ * kernels hand on to one another lives in a static device array of BMF_AGGREGATE_STATIC_MAX_DOUBLES doubles (32 MiB)
  * that every GPU loading this library holds until the process exits.
  *   mu:  device [J][R][K], Lam: device [J][R][K][K] (full symmetric precisions); submodel 0 is
  *        the one whose posterior was propagated to the others;
