@@ -123,8 +123,11 @@ typedef enum {
     BMF_E_STATE = 8      /* call not valid now (e.g. stage 2 before stage 1) */
 } bmf_status;
 
-/* Precision of the gathered factor copies and of the Gram accumulation.  The conditional
- * assembly, Cholesky, solves, draws, hyperparameter step and moments are FP64 in all modes.
+/* Precision of the gathered factor copies and of the Gram accumulation.  The
+ * hyperparameter step, moments and states are FP64 in all modes, and so are the conditional
+ * assembly, Cholesky, solves and draws, except that the reduced-precision modes take them in pairs
+ * of floats (48 bits, twice what their Gram sums carry) at 9 <= K <= 48, with FP64 for rows whose
+ * range or conditioning needs it.
  * FP32 gathers at K > 16 reach the tensor cores as split TF32 (three products per tile, close to
  * FP32 products); BMF_TF32 keeps FP32 gathers but takes one TF32 product per tile (operands
  * rounded to 10-bit mantissas) at K > 16, and is BMF_FP32 at K <= 16. */
@@ -258,7 +261,8 @@ typedef struct {
                           directly.  Ignored while profiling is on, and for a call given host
                           draws: their copy then runs in groups of sweeps beside the sweeps,
                           each sweep waiting only for its own group. */
-    int32_t cond_lanes; /* K >= 13: lanes that factor one row in the FP64 conditional draw (2, 4,
+    int32_t cond_lanes; /* K >= 13: lanes that factor one row in the FP64 conditional draw (ignored
+                          by the reduced-precision modes up to K = 48; 2, 4,
                           8, 16 or 32; every choice gives bit-identical values; 2, only for
                           K <= 16, keeps the row's matrix in registers; a team of 4 to 32 lanes
                           keeps it in shared memory, and bmf_set_schedule rejects a team whose

@@ -1053,7 +1053,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             cp.obs_val = me.val;
             cp.P = gp.P;
             cp.ldP = gp.ldP;
-            // lanes per row of the conditional: one thread per row below K = 13, a team above
+            // lanes per row of the FP64 conditional: one thread per row below K = 13, a team above
             const int team = K >= kTeamMinK
                                  ? (c->sched.cond_lanes > 0 ? c->sched.cond_lanes : cond_team_size(K))
                                  : 1;
@@ -1063,8 +1063,9 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
                 q.blocks = me.blocks + ba;
                 q.blk0 = me.stat0 + ba;
                 traced(c, sx, f == 0 ? K_COND_X : K_COND_W, 1, [&] {
+                    if (launch_cond_pairs(c->prec, q, (int)(bb - ba), c->sms, sx)) return;
                     // two lanes per row: the register-resident kernel where it exists
-                    if (team == 2 && launch_cond_pair(c->prec, q, (int)(bb - ba), sx)) return;
+                    if (team == 2 && launch_cond_pair(q, (int)(bb - ba), sx)) return;
                     if (team > 1)
                         launch_cond_team(c->prec, q, (int)(bb - ba), team, sx);
                     else
@@ -1983,8 +1984,8 @@ bmf_status bmf_autotune(bmf_ctx *c, int32_t stage, int32_t subset, int32_t sweep
         }
         s = run_all(cands);
     }
-    if (!s && K >= kTeamMinK) {
-        // lanes per row of the conditional (every choice gives bit-identical values)
+    if (!s && K >= kTeamMinK && (c->prec == BMF_FP64 || K > kPairsMaxK)) {
+        // lanes per row of the FP64 conditional (every choice gives bit-identical values)
         cands.clear();
         const std::vector<int> tries = K <= 16 ? std::vector<int>{2, 4, 8} : std::vector<int>{8, 16, 32};
         for (int lanes : tries)

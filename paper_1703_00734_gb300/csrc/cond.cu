@@ -314,11 +314,18 @@ static bool launch_cond_fixed(const CondParams &a, int n_blocks, cudaStream_t st
     case 3: cond_kernel_k<3, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
     case 4: cond_kernel_k<4, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
     case 5: cond_kernel_k<5, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
-    case 10: cond_kernel_k<10, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
-    case 11: cond_kernel_k<11, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
-    case 12: cond_kernel_k<12, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
-    default: return false;
+    default: break;
     }
+    // the reduced-precision modes draw K >= kPairsMinK in float pairs (cond_pairs.cu)
+    if constexpr (sizeof(GT) == 8) {
+        switch (a.K) {
+        case 10: cond_kernel_k<10, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
+        case 11: cond_kernel_k<11, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
+        case 12: cond_kernel_k<12, GT, AT><<<n_blocks, kCondBlock, 0, st>>>(a); return true;
+        default: break;
+        }
+    }
+    return false;
 }
 
 template <typename GT, typename AT>

@@ -1,4 +1,4 @@
-// cond_pair.cu -- the FP64 conditional draw of a row for 13 <= K <= 16 with the row's matrix in
+// cond_pair.cu -- the FP64 mode's conditional draw of a row for 13 <= K <= 16 with the row's matrix in
 // registers (the same draw as cond.cu and the team kernel of wide.cu: Eqs. 2-4,
 //   Lambda_n = Lambda_p + tau G_n, b_n = Lambda_p mu_p + tau r_n, Lambda_n = L L^T,
 //   x_n = L^{-T} (L^{-1} b_n + z_n)).
@@ -12,25 +12,14 @@
 // k of L reaches the other lane by shuffles.  Every entry sees the operations of the team kernel
 // in the same order (right-looking Cholesky, column-oriented solves), so the values are
 // bit-identical to it.  A row with few observations (kFusedRow) forms its own G_n and r_n from
-// its list and the gathered partner rows, each entry accumulated in list order in the Gram
-// pass's accumulation type, instead of reading Gram partials.
-#include <cuda_bf16.h>
-
+// its list and the gathered partner rows, each entry accumulated in list order, instead of
+// reading Gram partials.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace bmf {
 
 namespace {
-
-template <typename GT>
-__device__ __forceinline__ GT narrow_to(double x);
-template <>
-__device__ __forceinline__ double narrow_to<double>(double x) { return x; }
-template <>
-__device__ __forceinline__ float narrow_to<float>(double x) { return (float)x; }
-template <>
-__device__ __forceinline__ __nv_bfloat16 narrow_to<__nv_bfloat16>(double x) { return __double2bfloat16(x); }
 
 // Row of slot s of lane l, the lane owning row i, and the entries slot s can hold.
 __device__ __forceinline__ int pair_row(int s, int l) { return 2 * s + (l ^ (s & 1)); }
@@ -64,49 +53,21 @@ __device__ __forceinline__ void prefetch_wait() { asm volatile("cp.async.wait_al
 
 int cond_pair_smem(int K) { return kCondBlock * (ntri(K) + K) * (int)sizeof(double); }
 
-// The first K entries of a gathered partner row (16-byte aligned, at least the padded K
-// entries long) with vector loads, in the accumulation type of the Gram sums.
-template <int K, typename GT, typename AT>
-__device__ __forceinline__ void load_partner(const GT *__restrict__ p, AT (&w)[K])
+// The first K entries of a gathered partner row (16-byte aligned, at least the padded K entries
+// long) with vector loads.
+template <int K>
+__device__ __forceinline__ void load_partner(const double *__restrict__ p, double (&w)[K])
 {
-    if constexpr (sizeof(GT) == 8) {
-        const double2 *q = reinterpret_cast<const double2 *>(p);
+    const double2 *q = reinterpret_cast<const double2 *>(p);
 #pragma unroll
-        for (int c = 0; c < (K + 1) / 2; ++c) {
-            const double2 v = __ldg(q + c);
-            w[2 * c] = v.x;
-            if (2 * c + 1 < K) w[2 * c + 1] = v.y;
-        }
-    } else if constexpr (sizeof(GT) == 4) {
-        const float4 *q = reinterpret_cast<const float4 *>(p);
-#pragma unroll
-        for (int c = 0; c < (K + 3) / 4; ++c) {
-            const float4 v = __ldg(q + c);
-            const float f[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (4 * c + u < K) w[4 * c + u] = f[u];
-        }
-    } else {
-        const uint4 *q = reinterpret_cast<const uint4 *>(p);
-#pragma unroll
-        for (int c = 0; c < (K + 7) / 8; ++c) {
-            const uint4 v = __ldg(q + c);
-            const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u4[u]));
-                if (8 * c + 2 * u < K) w[8 * c + 2 * u] = f.x;
-                if (8 * c + 2 * u + 1 < K) w[8 * c + 2 * u + 1] = f.y;
-            }
-        }
+    for (int c = 0; c < (K + 1) / 2; ++c) {
+        const double2 v = __ldg(q + c);
+        w[2 * c] = v.x;
+        if (2 * c + 1 < K) w[2 * c + 1] = v.y;
     }
 }
 
-__device__ __forceinline__ float macc(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double macc(double a, double b, double c) { return fma(a, b, c); }
-
-template <int K, typename GT, typename AT>
+template <int K>
 __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
 {
     constexpr int S = (K + 1) / 2;
@@ -151,35 +112,35 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
     //      finite; they write nothing)
     if (active) {
         const double *hp = h >= 0 ? a.hyper + (int64_t)h * hyper_slot_len(K) : nullptr;
-        const AT *pp = static_cast<const AT *>(a.part) + (i0 - a.item0) * (int64_t)a.ld;
+        const double *pp = static_cast<const double *>(a.part) + (i0 - a.item0) * (int64_t)a.ld;
         const double *ps = mi >= 0 ? a.rowsum + (int64_t)mi * a.ld_sum : nullptr;
         if (mi == kFusedRow) {
             // a row with few observations: its Gram sums from its own list, each entry
             // accumulated in list order (the Gram pass skips the row)
-            AT G[S][K], Rv[S];
+            double G[S][K], Rv[S];
 #pragma unroll
             for (int s = 0; s < S; ++s) {
 #pragma unroll
-                for (int j = 0; j < slot_len(K, s); ++j) G[s][j] = AT(0);
-                Rv[s] = AT(0);
+                for (int j = 0; j < slot_len(K, s); ++j) G[s][j] = 0.0;
+                Rv[s] = 0.0;
             }
             const int no = (int)(o1 - o0);
             // observations in groups of four: indices and values first, then the partner rows
             constexpr int QG = 4;
             for (int c0 = 0; c0 < no; c0 += QG) {
                 int32_t pid[QG];
-                AT yv[QG];
+                double yv[QG];
 #pragma unroll
                 for (int q2 = 0; q2 < QG; ++q2)
                     if (c0 + q2 < no) {
                         pid[q2] = a.obs_idx[o0 + c0 + q2];
-                        yv[q2] = static_cast<const AT *>(a.obs_val)[o0 + c0 + q2];
+                        yv[q2] = static_cast<const double *>(a.obs_val)[o0 + c0 + q2];
                     }
 #pragma unroll
                 for (int q2 = 0; q2 < QG; ++q2)
                     if (c0 + q2 < no) {
-                        AT pv[K];
-                        load_partner<K, GT, AT>(static_cast<const GT *>(a.P) + (int64_t)pid[q2] * a.ldP,
+                        double pv[K];
+                        load_partner<K>(static_cast<const double *>(a.P) + (int64_t)pid[q2] * a.ldP,
                                                 pv);
 #pragma unroll
                         for (int s = 0; s < S; ++s) {
@@ -187,8 +148,8 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
                             if (i < K) {
 #pragma unroll
                                 for (int j = 0; j < slot_len(K, s); ++j)
-                                    if (j <= i) G[s][j] = macc(pv[i], pv[j], G[s][j]);
-                                Rv[s] = macc(yv[q2], pv[i], Rv[s]);
+                                    if (j <= i) G[s][j] = fma(pv[i], pv[j], G[s][j]);
+                                Rv[s] = fma(yv[q2], pv[i], Rv[s]);
                             }
                         }
                     }
@@ -202,10 +163,10 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
                         if (j <= i) {
                             const int e = tri(i, j);
                             const double prior = hp ? hp[K + e] : a.prior_L[(int64_t)e * R + r];
-                            M[s][j] = fma(tau, widen(G[s][j]), prior);
+                            M[s][j] = fma(tau, G[s][j], prior);
                         }
                     const double prior = hp ? hp[K + NT + i] : a.prior_b[(int64_t)i * R + r];
-                    B[s] = fma(tau, widen(Rv[s]), prior);
+                    B[s] = fma(tau, Rv[s], prior);
                 } else {
 #pragma unroll
                     for (int j = 0; j < slot_len(K, s); ++j) M[s][j] = 0.0;
@@ -221,12 +182,12 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
                     for (int j = 0; j < slot_len(K, s); ++j)
                         if (j <= i) {
                             const int e = tri(i, j);
-                            const double gsum = ps ? ps[e] : (i1 > i0 ? widen(pp[e]) : 0.0);
+                            const double gsum = ps ? ps[e] : (i1 > i0 ? pp[e] : 0.0);
                             const double prior = hp ? hp[K + e] : a.prior_L[(int64_t)e * R + r];
                             M[s][j] = fma(tau, gsum, prior);
                         }
                     const int src = a.part_rhs + i;
-                    const double gsum = ps ? ps[src] : (i1 > i0 ? widen(pp[src]) : 0.0);
+                    const double gsum = ps ? ps[src] : (i1 > i0 ? pp[src] : 0.0);
                     const double prior = hp ? hp[K + NT + i] : a.prior_b[(int64_t)i * R + r];
                     B[s] = fma(tau, gsum, prior);
                 } else {
@@ -251,7 +212,7 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
     for (int k = 0; k < K; ++k) {
         const double d = __shfl_sync(kFull, M[k / 2][k], pb + pair_owner(k));
         if (!pivot_ok(d)) ok = false;
-        const double rs = ok ? pivot_rsqrt<GT>(d) : 0.0;
+        const double rs = ok ? rsqrt(d) : 0.0;
         if (l == pair_owner(k)) RI[k / 2] = rs;
 #pragma unroll
         for (int s = 0; s < S; ++s)
@@ -318,17 +279,17 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
     for (int j = 0; j < K; ++j) xall[j] = __shfl_sync(kFull, B[j / 2], pb + pair_owner(j));
     if (moments) prefetch_wait();
     if (active && ok) {
-        GT *g = static_cast<GT *>(a.Xg) + r * a.ldg;
+        double *g = static_cast<double *>(a.Xg) + r * a.ldg;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             const int i = pair_row(s, l);
             if (i < K) {
                 a.X[r * K + i] = B[s];
-                g[i] = narrow_to<GT>(B[s]);
+                g[i] = B[s];
                 if (a.keep) a.S1[(int64_t)i * R + r] = mine[NT + i] + B[s];
             }
         }
-        for (int i = K + l; i < a.ldg; i += 2) g[i] = narrow_to<GT>(0.0);
+        for (int i = K + l; i < a.ldg; i += 2) g[i] = 0.0;
         if (a.keep && a.full) {
 #pragma unroll
             for (int s = 0; s < S; ++s) {
@@ -363,34 +324,30 @@ __global__ void __launch_bounds__(kPairThreads) cond_pair_kernel(CondParams a)
     }
 }
 
-template <int K, typename GT, typename AT>
+template <int K>
 static void launch_pair_k(const CondParams &a, int n_blocks, cudaStream_t st)
 {
     const int smem = a.keep ? cond_pair_smem(K) : 0;
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(cond_pair_kernel<K, GT, AT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(cond_pair_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              cond_pair_smem(K));
-    cond_pair_kernel<K, GT, AT><<<n_blocks, kPairThreads, smem, st>>>(a);
+    cond_pair_kernel<K><<<n_blocks, kPairThreads, smem, st>>>(a);
 }
 
-template <typename GT, typename AT>
 static bool launch_pair_t(const CondParams &a, int n_blocks, cudaStream_t st)
 {
     switch (a.K) {
-    case 13: launch_pair_k<13, GT, AT>(a, n_blocks, st); return true;
-    case 14: launch_pair_k<14, GT, AT>(a, n_blocks, st); return true;
-    case 15: launch_pair_k<15, GT, AT>(a, n_blocks, st); return true;
-    case 16: launch_pair_k<16, GT, AT>(a, n_blocks, st); return true;
+    case 13: launch_pair_k<13>(a, n_blocks, st); return true;
+    case 14: launch_pair_k<14>(a, n_blocks, st); return true;
+    case 15: launch_pair_k<15>(a, n_blocks, st); return true;
+    case 16: launch_pair_k<16>(a, n_blocks, st); return true;
     default: return false;
     }
 }
 
-bool launch_cond_pair(int prec, const CondParams &a, int n_blocks, cudaStream_t st)
+bool launch_cond_pair(const CondParams &a, int n_blocks, cudaStream_t st)
 {
-    if (n_blocks <= 0) return true;
-    if (prec == BMF_FP64) return launch_pair_t<double, double>(a, n_blocks, st);
-    if (prec == BMF_FP32) return launch_pair_t<float, float>(a, n_blocks, st);
-    return launch_pair_t<__nv_bfloat16, float>(a, n_blocks, st);
+    return n_blocks <= 0 || launch_pair_t(a, n_blocks, st);
 }
 
 }  // namespace bmf

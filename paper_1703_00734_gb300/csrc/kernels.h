@@ -92,6 +92,10 @@ struct CondParams {
     int ldP;
 };
 void launch_cond(int prec, const CondParams &a, int n_blocks, cudaStream_t st);
+// The draw in float pairs for the reduced-precision modes at kPairsMinK <= K <= kPairsMaxK
+// (cond_pairs.cu).  False for the others (nothing launched).
+constexpr int kPairsMinK = 9, kPairsMaxK = 48;
+bool launch_cond_pairs(int prec, const CondParams &a, int n_blocks, int sms, cudaStream_t st);
 // multi_idx of a row whose Gram sums the conditional draw forms itself: 13 <= K <= 16 (the
 // two-lane and team conditionals) and 1 to kFuseMaxObs observations in one work item.  Such a
 // row's partner rows are few and mostly cached, where its Gram partials would be a round trip
@@ -280,7 +284,7 @@ int cond_team_size(int K);
 bool cond_lanes_valid(int K, int lanes);
 // The same draw for 13 <= K <= 16 with two lanes per row and the row's matrix in registers
 // (cond_pair.cu; bit-identical to the team kernel).  False for other K (nothing launched).
-bool launch_cond_pair(int prec, const CondParams &a, int n_blocks, cudaStream_t st);
+bool launch_cond_pair(const CondParams &a, int n_blocks, cudaStream_t st);
 
 // Adjoint of the masked log-joint (adjoint.cu).
 int adjoint_kt(int K);          // template width (K rounded up to 4, 8, 12, 16, 32 or 64)
