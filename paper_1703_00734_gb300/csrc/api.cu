@@ -163,6 +163,7 @@ struct bmf_ctx {
     double *gen_d = nullptr;
     int64_t gen_cap = 0;
     GenSeg *gen_segs_d = nullptr;
+    GenTables *gen_tab = nullptr;
     int64_t gen_segs_cap = 0;
     double *aggX = nullptr, *aggW = nullptr;   // aggregated means, reordered order
     unsigned long long *ncorr_d = nullptr;
@@ -613,7 +614,6 @@ bmf_status prepare_gen(bmf_ctx *c, int sl0, int sl1, int64_t per, int nbuf, int6
     *n_segs = (int)segs.size();
     if ((int64_t)segs.size() > c->gen_segs_cap) {
         if (c->gen_segs_d) cudaFree(c->gen_segs_d);
-    if (c->pred_buf) cudaFree(c->pred_buf);
         c->gen_segs_d = nullptr;
         c->gen_segs_cap = 0;
         if (cudaMalloc(&c->gen_segs_d, segs.size() * sizeof(GenSeg)) != cudaSuccess)
@@ -638,7 +638,7 @@ bmf_status prepare_gen(bmf_ctx *c, int sl0, int sl1, int64_t per, int nbuf, int6
 
 void enqueue_gen(bmf_ctx *c, int64_t units, int n_segs, int64_t t, double *out)
 {
-    GenParams gp{c->gen_segs_d, n_segs, units, c->seed, t, out, c->W.ptr, c->err_d};
+    GenParams gp{c->gen_segs_d, n_segs, units, c->seed, t, out, c->W.ptr, c->err_d, c->gen_tab};
     traced(c, c->st, K_GEN, 1, [&] { launch_gen(gp, c->st); });
 }
 
@@ -1123,7 +1123,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
         }
         if (tail_gen) {
             GenParams gp{c->gen_segs_d, gen_segs, gen_units, c->seed, t + 2,
-                         c->gen_d + (int64_t)(it & 1) * per, c->W.ptr, c->err_d};
+                         c->gen_d + (int64_t)(it & 1) * per, c->W.ptr, c->err_d, c->gen_tab};
             traced(c, c->st5, K_GEN, 1, [&] { launch_gen(gp, c->st5); });
             CUDA_TRY(c, cudaEventRecord(c->ev_gen[it & 1], c->st5));
         }
@@ -1701,6 +1701,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     c->rmse_part = c->mem.alloc<double>(2 * c->rmse_blocks);
     c->rmse_out = c->mem.alloc<double>(2);
     c->err_d = c->mem.alloc<DevError>(1);
+    c->gen_tab = c->mem.alloc<GenTables>(1);
     c->aggX = c->mem.alloc<double>(N * K);
     c->aggW = c->mem.alloc<double>(D * K);
     c->ncorr_d = c->mem.alloc<unsigned long long>(1);
@@ -1753,6 +1754,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     }
     DevError z = {0u, INT32_MAX};
     cudaMemcpy(c->err_d, &z, sizeof(z), cudaMemcpyHostToDevice);
+    cudaMemcpy(c->gen_tab, &gen_tables(), sizeof(GenTables), cudaMemcpyHostToDevice);
     // aggregation bases: X block i over submodels (i, j), then W block j over (i, j)
     {
         std::vector<int64_t> base((size_t)(I + J) * MB, 0);

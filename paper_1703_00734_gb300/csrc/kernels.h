@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "rng_tables.h"
 
 namespace bmf {
 
@@ -340,6 +341,7 @@ struct GenParams {
     double *out;
     const int64_t *cnt_ptr;   // kind 4: W arena observation offsets (entries of a column)
     DevError *err;
+    const GenTables *tab;     // device copy of gen_tables()
 };
 struct GenSubset {
     int32_t sid;
