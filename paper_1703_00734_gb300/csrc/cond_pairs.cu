@@ -18,7 +18,7 @@
 // the FP32 gathers of ill-conditioned rows, to more than 2e-5 of the posterior means within ten
 // sweeps (50,000 x 12,500, K = 64, sigma 0.3: 5e-5, half of what FP32 gathers are off by).
 //
-// A row whose terms leave the range of a pair, or whose pivot loses 32 bits to cancellation (among
+// A row whose terms leave the range of a pair, or whose pivot loses 20 bits to cancellation (among
 // them every row that is not positive definite), is redone in FP64 by cond_row_serial, so what
 // is accepted and what is rejected is decided in FP64.
 #include <algorithm>
@@ -114,8 +114,8 @@ __device__ __noinline__ bool cond_row_serial(const CondParams &a, int64_t r, dou
     return true;
 }
 
-// A pivot that lost 32 of its 48 bits (or is not positive, or NaN) sends its row to FP64.
-constexpr float kPivotLoss = 0x1p-32f;
+// A pivot that lost 20 of its 48 bits (or is not positive, or NaN) sends its row to FP64.
+constexpr float kPivotLoss = 0x1p-20f;
 
 }  // namespace
 
