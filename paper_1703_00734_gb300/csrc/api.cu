@@ -207,6 +207,7 @@ struct bmf_ctx {
     double *ring[2] = {nullptr, nullptr};
     double *mix[2] = {nullptr, nullptr};
     int8_t *has_mix[2] = {nullptr, nullptr};
+    int32_t *sum_over = nullptr, *sum_over_n = nullptr;   // scratch of one summary launch
     // adjoint / Langevin scratch (allocated on first use)
     float *adj_part = nullptr;
     int64_t adj_part_cap = 0;
@@ -1235,8 +1236,10 @@ bmf_status finalize_subset(bmf_ctx *c, int sid)
             sp.mm_b = sd.mm_b;
             sp.mix = c->summary == BMF_SUMMARY_GMM ? c->mix[f] : nullptr;
             sp.R = sd.R;
+            sp.over = c->sum_over;
+            sp.over_n = c->sum_over_n;
             sp.err = c->err_d;
-            launch_summary(sp, c->st);
+            CUDA_TRY(c, launch_summary(sp, c->st));
         }
         su.finalized = true;
         return BMF_OK;
@@ -1733,6 +1736,10 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
         c->noise_blocks = c->mem.alloc<NoiseBlock>(S);
         if (c->mem.ok && nx)
             cudaMemcpy(c->xval_orig, c->X.val, (size_t)nx * vb, cudaMemcpyDeviceToDevice);
+    }
+    if (c->summary != BMF_SUMMARY_MM) {
+        c->sum_over = c->mem.alloc<int32_t>(std::max(N, D));
+        c->sum_over_n = c->mem.alloc<int32_t>(1);
     }
     if (c->summary != BMF_SUMMARY_MM)
         for (int f = 0; f < 2; ++f) {
@@ -2654,8 +2661,8 @@ bmf_status bmf_fit_summaries(int32_t K, int64_t R, int32_t S, const double *samp
     }
     if (R == 0) return BMF_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    DevError *err = nullptr;
-    if (cudaMalloc(&err, sizeof(DevError)) != cudaSuccess) {
+    DevError *err = nullptr;   // the error word, then the list of rows with many clusters
+    if (cudaMalloc(&err, sizeof(DevError) + (size_t)(R + 1) * sizeof(int32_t)) != cudaSuccess) {
         g_init_error = "bmf_fit_summaries: device allocation failed";
         return BMF_E_OOM;
     }
@@ -2678,11 +2685,10 @@ bmf_status bmf_fit_summaries(int32_t K, int64_t R, int32_t S, const double *samp
     sp.pooled_Lam = pooled_Lam;
     sp.assign = assign;
     sp.R = R;
+    sp.over_n = reinterpret_cast<int32_t *>(err + 1);
+    sp.over = sp.over_n + 1;
     sp.err = err;
-    if (e == cudaSuccess) {
-        launch_summary(sp, st);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = launch_summary(sp, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, sizeof h, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(err);

@@ -231,9 +231,9 @@ void launch_predict_sq(const PredictParams &p, int blocks, cudaStream_t st);
 void launch_gather_rows(int K, int64_t R, const int64_t *src, const double *in, double *out,
                         cudaStream_t st);
 
-// Summaries beyond moment matching (summary.cu; Section 4.1 PP DM / PP GMM): one warp per row
-// clusters the row's retained samples by lambda-means and fits the dominant mode (mode 1), the
-// C largest modes (mode 2) or all samples (mode 0), with the pooled moments of the mixture.
+// Summaries beyond moment matching (summary.cu; Section 4.1 PP DM / PP GMM): every row's retained
+// samples clustered by lambda-means, and Gaussian fits of the dominant mode (mode 1), the C
+// largest modes (mode 2) or all samples (mode 0), with the pooled moments of the mixture.
 constexpr int kMaxComponents = 4;
 struct SummaryParams {
     int K, S, C, mode;
@@ -251,10 +251,10 @@ struct SummaryParams {
     // [R][C][1 + 2K + ntri(K)] (score constant, mean, packed precision, precision x mean)
     double *mm_mu, *mm_L, *mm_b, *mix;
     int64_t R;
+    int32_t *over, *over_n;    // scratch: [n_rows] rows that open many clusters, their number
     DevError *err;
 };
-size_t summary_smem(int K, int S);
-void launch_summary(const SummaryParams &p, cudaStream_t st);
+cudaError_t launch_summary(const SummaryParams &p, cudaStream_t st);
 
 // Component choice of a propagated mixture prior for arena rows [r0, r0 + n) that carry one
 // (has_mix): the component with the largest responsibility at the current X becomes the row's

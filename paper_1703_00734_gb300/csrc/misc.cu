@@ -470,10 +470,6 @@ void launch_rmse_final(const double *partial, int blocks, double *out2, cudaStre
 
 // ------------------------------------------------------------------------------------------
 // Moment matching: mu = S1/S, Sigma = S2/S - mu mu^T, Lambda = Sigma^{-1}, b = Lambda mu.
-// Sigma = L L^T in place, then W = L^{-1} in place (columns left to right; W_ij =
-// -(1/L_ii) sum_{k=j}^{i-1} L_ik W_kj reads only entries of L right of column j and entries of W
-// already written), then Lambda = W^T W in place (rows top to bottom through a K-vector: row i
-// of Lambda needs only rows k >= i of W), then b.  K^3/2 multiply-adds and no division.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kRowBlock) mm_kernel(MMParams a)
 {
@@ -491,27 +487,10 @@ __global__ void __launch_bounds__(kRowBlock) mm_kernel(MMParams a)
         for (int j = 0; j <= i; ++j)
             RS(A, tri(i, j)) = fma(-mi, RS(mu, j), a.S2[(int64_t)tri(i, j) * R + r] * inv);
     }
-    if (!row_chol(A, v, K, rb)) {
+    if (!row_spd_inverse(A, v, K, rb, nullptr)) {
         atomicOr(&a.err->flags, ERR_NOT_PD);
         atomicMin(&a.err->first_bad_row, (int)r);
         return;
-    }
-    for (int j = 0; j < K; ++j) {
-        RS(A, tri(j, j)) = RS(v, j);
-        for (int i = j + 1; i < K; ++i) {
-            const int ii = tri(i, 0);
-            double s = 0.0;
-            for (int k = j; k < i; ++k) s = fma(RS(A, ii + k), RS(A, tri(k, j)), s);
-            RS(A, ii + j) = -s * RS(v, i);
-        }
-    }
-    for (int i = 0; i < K; ++i) {
-        for (int j = 0; j <= i; ++j) {
-            double s = 0.0;
-            for (int k = i; k < K; ++k) s = fma(RS(A, tri(k, i)), RS(A, tri(k, j)), s);
-            RS(v, j) = s;
-        }
-        for (int j = 0; j <= i; ++j) RS(A, tri(i, j)) = RS(v, j);
     }
     for (int i = 0; i < K; ++i) a.mu[r * K + i] = RS(mu, i);
     for (int e = 0; e < NT; ++e) a.L[(int64_t)e * R + r] = RS(A, e);

@@ -57,6 +57,39 @@ static __device__ void row_solve(const double *P, const double *ri, double *v, i
     }
 }
 
+// Inverse of the packed SPD matrix A in place; v: K scratch slots.  A = L L^T in place, then
+// W = L^{-1} in place (columns left to right; W_ij = -(1/L_ii) sum_{k=j}^{i-1} L_ik W_kj reads only
+// entries of L right of column j and entries of W already written), then A^{-1} = W^T W in place
+// (rows top to bottom through v: row i needs only rows k >= i of W).  K^3/2 multiply-adds and no
+// division.  logdet (nullable): log det(A^{-1}) / 2 = sum log(1 / L_ii).  False if a pivot is not > 0.
+static __device__ bool row_spd_inverse(double *A, double *v, int K, int rb, double *logdet)
+{
+    if (!row_chol(A, v, K, rb)) return false;
+    if (logdet) {
+        double s = 0.0;
+        for (int i = 0; i < K; ++i) s += log(RS(v, i));
+        *logdet = s;
+    }
+    for (int j = 0; j < K; ++j) {
+        RS(A, tri(j, j)) = RS(v, j);
+        for (int i = j + 1; i < K; ++i) {
+            const int ii = tri(i, 0);
+            double s = 0.0;
+            for (int k = j; k < i; ++k) s = fma(RS(A, ii + k), RS(A, tri(k, j)), s);
+            RS(A, ii + j) = -s * RS(v, i);
+        }
+    }
+    for (int i = 0; i < K; ++i) {
+        for (int j = 0; j <= i; ++j) {
+            double s = 0.0;
+            for (int k = i; k < K; ++k) s = fma(RS(A, tri(k, i)), RS(A, tri(k, j)), s);
+            RS(v, j) = s;
+        }
+        for (int j = 0; j <= i; ++j) RS(A, tri(i, j)) = RS(v, j);
+    }
+    return true;
+}
+
 // In-place packed lower Cholesky used only as a positive-definiteness test (pivot > 0 at every
 // step), scaling by one reciprocal per column.
 static __device__ bool row_pd_test(double *P, int K, int rb)

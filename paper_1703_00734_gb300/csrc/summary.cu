@@ -1,11 +1,13 @@
 // summary.cu -- the subset-posterior summaries beyond moment matching (Section 4.1, "PP DM"
 // and "PP GMM"; Section 5.1) and the component choice of a propagated mixture prior.
 //
-//   * summary_kernel: one warp per row clusters the row's retained samples by lambda-means and
-//     fits Gaussians to the largest clusters (dominant mode: the largest one; mixture: the C
-//     largest with at least K + 1 samples, weighted by their sizes; a row without such a
-//     cluster falls back to one Gaussian over all samples), then the mixture's pooled mean and
-//     covariance, which Eq. 14 aggregates (Section 4.2).
+//   * cluster_kernel: one warp per row clusters the row's retained samples by lambda-means and
+//     forms the means and covariances of the largest clusters (dominant mode: the largest one;
+//     mixture: the C largest with at least K + 1 samples, weighted by their sizes);
+//   * fit_kernel: one thread per row takes their precisions (a row without such a cluster falls
+//     back to one Gaussian over all samples) and the mixture's pooled mean and covariance, which
+//     Eq. 14 aggregates (Section 4.2).  20,000 rows of 200 samples at K = 10, three modes:
+//     21.0 ms with one warp per row for everything, 2.2 ms with these;
 //   * mix_choose_kernel: one thread per row picks, before each draw, the component with the
 //     largest responsibility pi_c N(x; mu_c, Lambda_c^{-1}) at the row's current value and
 //     installs it as the row's prior.
@@ -18,12 +20,14 @@
 // until no assignment changes (at most 100).  The warp scores the samples in parallel against
 // the existing centres, then walks the samples in order to open new clusters, updating the
 // later samples' nearest centre after each opening: the same assignments as the sequential
-// visit.  Every sum runs over the samples in order with separate multiplies and adds, so
-// assignments and fits do not depend on the launch shape.
+// visit.  Every sum runs over the samples in order, so assignments and fits do not depend on the
+// launch shape.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "rows.cuh"
 
 namespace bmf {
 
@@ -46,401 +50,479 @@ __device__ double sqdist(const double *p, const double *c, int K)
     return d;
 }
 
-// Lower Cholesky factor of the K x K row-major matrix A into L (warp; lane i computes row i
-// below the pivot, each entry summed in order); false if a pivot is not > 0.
-__device__ bool warp_chol(const double *A, double *L, int K, int lane)
+// The same in FP32 from rounded vectors.
+__device__ float sqdist32(const float *p, const float *c, int K)
 {
-    for (int e = lane; e < K * K; e += 32) L[e] = 0.0;
-    __syncwarp();
-    for (int j = 0; j < K; ++j) {
-        double d = 0.0;
-        if (lane == 0) {
-            double s = A[j * K + j];
-            for (int k = 0; k < j; ++k) s = dsub(s, dmul(L[j * K + k], L[j * K + k]));
-            d = s > 0.0 ? sqrt(s) : -1.0;
-            if (s > 0.0) L[j * K + j] = d;
-        }
-        d = __shfl_sync(kAll, d, 0);
-        if (!(d > 0.0)) return false;
-        __syncwarp();
-        for (int i = j + 1 + lane; i < K; i += 32) {
-            double t = A[i * K + j];
-            for (int k = 0; k < j; ++k) t = dsub(t, dmul(L[i * K + k], L[j * K + k]));
-            L[i * K + j] = t / d;
-        }
-        __syncwarp();
+    float d = 0.f;
+    for (int k = 0; k < K; ++k) {
+        const float e = p[k] - c[k];
+        d = fmaf(e, e, d);
     }
-    return true;
+    return d;
 }
 
-// Inverse of the SPD matrix A (K x K) into Ainv from its Cholesky factor L: lane j solves
-// L L^T x = e_j (forward then back substitution, in order), then the two triangles are
-// averaged.  col: K * 32 scratch (a column per lane).
-__device__ bool warp_spd_inverse(const double *A, double *Ainv, double *L, double *col, int K,
-                                 int lane)
+// Where the fits of a row pass between the two kernels: sizes, means and packed lower covariances
+// of up to C components, inside the arrays that end up holding the results.  Row index q is
+// row - row0 (fit outputs) or the arena row (library layout).
+struct FitStage {
+    double *n, *m, *S;
+    int64_t n_row, n_c, m_row, m_c, S_row, S_c, S_e;
+    __device__ double &size(int64_t q, int c) const { return n[q * n_row + c * n_c]; }
+    __device__ double &mean(int64_t q, int c, int k) const { return m[q * m_row + c * m_c + k]; }
+    __device__ double &cov(int64_t q, int c, int e) const { return S[q * S_row + c * S_c + e * S_e]; }
+};
+
+__host__ __device__ FitStage fit_stage(const SummaryParams &p)
 {
-    if (!warp_chol(A, L, K, lane)) return false;
-    for (int j = lane; j < K; j += 32) {
-        double *y = col + (size_t)lane * K;
-        for (int i = 0; i < K; ++i) y[i] = i == j ? 1.0 : 0.0;
-        for (int i = 0; i < K; ++i) {
-            double t = y[i];
-            for (int k = 0; k < i; ++k) t = dsub(t, dmul(L[i * K + k], y[k]));
-            y[i] = t / L[i * K + i];
-        }
-        for (int i = K - 1; i >= 0; --i) {
-            double t = y[i];
-            for (int k = i + 1; k < K; ++k) t = dsub(t, dmul(L[k * K + i], y[k]));
-            y[i] = t / L[i * K + i];
-        }
-        for (int i = 0; i < K; ++i) Ainv[i * K + j] = y[i];
-    }
-    __syncwarp();
-    for (int e = lane; e < K * K; e += 32) {
-        const int i = e / K, j = e % K;
-        if (j < i) {
-            const double m = dmul(0.5, dadd(Ainv[i * K + j], Ainv[j * K + i]));
-            Ainv[i * K + j] = m;
-            Ainv[j * K + i] = m;
-        }
-    }
-    __syncwarp();
-    return true;
+    const int64_t K = p.K, C = p.C, KK = K * K, W = 1 + 2 * K + K * (K + 1) / 2;
+    if (p.pi) return FitStage{p.pi, p.mu, p.Lam, C, 1, C * K, K, C * KK, KK, 1};
+    if (p.mix) return FitStage{p.mix, p.mix + 1, p.mix + 1 + K, C * W, W, C * W, W, C * W, W, 1};
+    return FitStage{p.mm_b, p.mm_mu, p.mm_L, 1, 0, K, 0, 1, 0, p.R};   // one component
+}
+
+constexpr int kFastCentres = 32;
+
+// Shared memory of one row (one warp) with at most `cap` clusters at a time (S of them survive a
+// round); fast: with FP32 copies of samples and centres.
+size_t cluster_smem(int K, int S, int cap, bool fast)
+{
+    const size_t centres = (size_t)std::min(cap, std::max(S, 1));
+    return ((size_t)S + centres) * K * (sizeof(double) + (fast ? sizeof(float) : 0)) +
+           (size_t)S * (sizeof(float) + 4 * sizeof(int)) + (2 * (size_t)cap + centres + 1) * sizeof(int);
 }
 
 }  // namespace
 
-// Shared memory of one row (one warp): samples, centres (at most 2S + 1), per-sample state and
-// the fit workspace (which reuses the centre area after the clustering): component means and
-// precisions, four K x K work matrices, a column per lane and the pooled mean.
-__host__ __device__ static size_t fit_doubles(int K)
-{
-    return (size_t)kMaxComponents * K + (size_t)kMaxComponents * K * K + (size_t)4 * K * K +
-           (size_t)32 * K + K;
-}
-
-size_t summary_smem(int K, int S)
-{
-    const size_t cen = (size_t)(2 * S + 1) * K;
-    const size_t fit = fit_doubles(K);
-    return ((size_t)S * K + (cen > fit ? cen : fit) + S) * sizeof(double) +
-           (size_t)(3 * S + 2 * (2 * S + 1) + 4) * sizeof(int);
-}
-
-__global__ void __launch_bounds__(32) summary_kernel(SummaryParams p)
+// lambda-means of one row per warp and the covariances of its chosen clusters.  FAST rows keep at
+// most kFastCentres clusters; rows that open more are listed for a second launch with room for
+// every sample's own (2 S + 1 within a round: a centre opened in the round is its sample).
+//
+// The distances decide only comparisons (which centre is nearest, whether it is beyond lambda):
+// FAST takes them in FP32, and again in FP64 where the FP32 values are closer than their error
+// bound, so the assignments are those of the FP64 procedure at a fraction of its FP64 work (a
+// warp's FP64 instruction takes 17 clocks of an SM, an FP32 one a quarter).  Centre means and
+// covariances run over member lists in sample order.
+template <bool FAST>
+__global__ void __launch_bounds__(32) cluster_kernel(SummaryParams p, int cap, const int32_t *list,
+                                                     const int32_t *list_n, int32_t *over, int32_t *over_n)
 {
     extern __shared__ double sh[];
     const int lane = threadIdx.x;
-    const int64_t row = blockIdx.x;
-    const int K = p.K, S = p.S, C = p.C;
-    const size_t cen_n = (size_t)(2 * S + 1) * K, fit_n = fit_doubles(K);
-    double *X = sh;                                   // [S][K]
-    double *cen = X + (size_t)S * K;                  // [2S+1][K] (clustering), fit area after
-    double *dbest = cen + (cen_n > fit_n ? cen_n : fit_n);   // [S]
-    int *assign = reinterpret_cast<int *>(dbest + S);        // [S]
-    int *prev = assign + S;                                  // [S]
-    int *best = prev + S;                                    // [S]
-    int *cnt = best + S;                                     // [2S+1]
-    int *map = cnt + 2 * S + 1;                              // [2S+1]
-    int *misc = map + 2 * S + 1;                             // [4]
-    for (int e = lane; e < S * K; e += 32) {
-        const int s = e / K, k = e % K;
-        X[e] = p.samples[(int64_t)s * p.sample_stride + (p.row0 + row) * K + k];
-    }
-    __syncwarp();
-    // ---- lambda-means ---------------------------------------------------------------------
-    int n = 0;
-    if (p.mode != 0 && S > 0) {
-        n = 1;
-        for (int k = lane; k < K; k += 32) cen[k] = X[k];
-        for (int i = lane; i < S; i += 32) prev[i] = -1;
+    const int K = p.K, S = p.S, C = p.C, NT = K * (K + 1) / 2, centres = min(cap, max(S, 1));
+    double *X = sh;                                              // [S][K]
+    double *cen = X + (size_t)S * K;                             // [centres][K]
+    float *Xf = reinterpret_cast<float *>(cen + (size_t)centres * K);   // [S][K] (FAST)
+    float *cenf = Xf + (FAST ? (size_t)S * K : 0);               // [centres][K] (FAST)
+    float *dbf = cenf + (FAST ? (size_t)centres * K : 0);        // [S] FP32 distance to the nearest
+    int *assign = reinterpret_cast<int *>(dbf + S);              // [S]
+    int *prev = assign + S;                                      // [S]
+    int *far = prev + S;                                         // [S] nearest is beyond lambda
+    int *member = far + S;                                       // [S] samples by cluster, in order
+    int *opened = member;                                        // before that: samples of the round's new centres
+    int *cnt = member + S, *map = cnt + cap, *off = map + cap;   // [cap], [cap], [centres + 1]
+    const FitStage fs = fit_stage(p);
+    const int64_t n_work = list ? (int64_t)*list_n : p.n_rows;
+    for (int64_t w = blockIdx.x; w < n_work; w += gridDim.x) {
+        const int64_t row = list ? list[w] : w;
         __syncwarp();
-        for (int it = 0; it < 100; ++it) {
-            // nearest existing centre of every sample (lowest index on ties)
-            for (int i = lane; i < S; i += 32) {
-                int b = 0;
-                double db = INFINITY;
-                for (int c = 0; c < n; ++c) {
-                    const double d = sqdist(X + (size_t)i * K, cen + (size_t)c * K, K);
-                    if (d < db) {
-                        db = d;
-                        b = c;
-                    }
-                }
-                best[i] = b;
-                dbest[i] = db;
+        float big = 0.f;
+        for (int e = lane; e < S * K; e += 32) {
+            const int s = e / K, k = e % K;
+            const double v = p.samples[(int64_t)s * p.sample_stride + (p.row0 + row) * K + k];
+            X[e] = v;
+            if constexpr (FAST) {
+                Xf[e] = (float)v;
+                big = fmaxf(big, fabsf((float)v));
             }
-            __syncwarp();
-            // samples in order: the next one farther than lambda from every centre opens a
-            // cluster; the later samples then compare with the new centre too
-            int pos = 0;
-            while (pos < S) {
-                int found = S;
-                for (int base = pos; base < S && found == S; base += 32) {
-                    const int i = base + lane;
-                    const unsigned v = __ballot_sync(kAll, i < S && dbest[i] > p.lambda);
-                    if (v) found = base + __ffs(v) - 1;
-                }
-                if (found == S) break;
-                const int c = n++;
-                for (int k = lane; k < K; k += 32) cen[(size_t)c * K + k] = X[(size_t)found * K + k];
-                if (lane == 0) best[found] = c;
-                __syncwarp();
-                for (int j = found + 1 + lane; j < S; j += 32) {
-                    const double d = sqdist(X + (size_t)j * K, cen + (size_t)c * K, K);
-                    if (d < dbest[j]) {
-                        dbest[j] = d;
-                        best[j] = c;
-                    }
-                }
-                __syncwarp();
-                pos = found + 1;
-            }
-            for (int i = lane; i < S; i += 32) assign[i] = best[i];
-            for (int c = lane; c < n; c += 32) cnt[c] = 0;
-            __syncwarp();
-            for (int i = lane; i < S; i += 32) atomicAdd(&cnt[assign[i]], 1);
-            __syncwarp();
-            if (lane == 0) {
-                int m = 0;
-                for (int c = 0; c < n; ++c) map[c] = cnt[c] > 0 ? m++ : -1;
-                misc[0] = m;
-            }
-            __syncwarp();
-            // centres to the means of their samples (in order), compacted in place: the new
-            // index never exceeds the old one and the sums read only the samples
-            for (int e = lane; e < n * K; e += 32) {
-                const int c = e / K, k = e % K;
-                if (map[c] < 0) continue;
-                double s = 0.0;
-                for (int i = 0; i < S; ++i)
-                    if (assign[i] == c) s = dadd(s, X[(size_t)i * K + k]);
-                cen[(size_t)map[c] * K + k] = s / (double)cnt[c];
-            }
-            __syncwarp();
-            n = misc[0];
-            int changed = 0;
-            for (int i = lane; i < S; i += 32) {
-                const int a = map[assign[i]];
-                assign[i] = a;
-                changed |= a != prev[i];
-                prev[i] = a;
-            }
-            __syncwarp();
-            if (!__any_sync(kAll, changed)) break;
         }
-    }
-    // cluster sizes under the final numbering
-    if (p.mode != 0 && S > 0) {
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) big = fmaxf(big, __shfl_xor_sync(kAll, big, o));
         __syncwarp();
-        for (int c = lane; c < n; c += 32) cnt[c] = 0;
-        __syncwarp();
-        for (int i = lane; i < S; i += 32) atomicAdd(&cnt[assign[i]], 1);
-        __syncwarp();
-    }
-    if (p.assign)
-        for (int i = lane; i < S; i += 32) p.assign[row * S + i] = p.mode != 0 ? assign[i] : 0;
-    // ---- fits -----------------------------------------------------------------------------
-    double *fmu = cen;                       // [C][K] component means
-    double *cL = fmu + (size_t)kMaxComponents * K;    // [C][K][K] component precisions
-    double *Sig = cL + (size_t)kMaxComponents * K * K;   // [K][K]
-    double *Lw = Sig + (size_t)K * K;        // [K][K]
-    double *Lam = Lw + (size_t)K * K;        // [K][K] current component precision
-    double *Acc = Lam + (size_t)K * K;       // [K][K] pooled covariance
-    double *col = Acc + (size_t)K * K;       // [32][K]
-    double *pm = col + (size_t)32 * K;       // [K] pooled mean
-    // the chosen clusters, largest first (ties: lowest index), written by lane 0
-    int *chosen = best;                      // [C] cluster ids, -1 unused
-    int *sizes = cnt;
-    int used = 0;
-    __syncwarp();
-    if (lane == 0) {
+        // Error of an FP32 squared distance d of rounded vectors with entries up to `big` (a mean
+        // of samples is no larger): each difference is off by at most eta = 2^-22 big, so d by at
+        // most 2 eta sqrt(K d) + K eta^2 + (K + 3) 2^-23 d; twice that is allowed for.
+        const float eta = 0x1p-22f * big;
+        auto slack = [&](float d) {
+            return 2.f * (2.f * eta * sqrtf(K * d) + K * eta * eta + (K + 3) * 0x1p-23f * d) + 1e-36f;
+        };
+        const float lamf = (float)p.lambda;
+        int n = 0;
+        bool too_many = false;
+        if (p.mode != 0 && S > 0) {
+            n = 1;
+            for (int k = lane; k < K; k += 32) {
+                cen[k] = X[k];
+                if constexpr (FAST) cenf[k] = Xf[k];
+            }
+            for (int i = lane; i < S; i += 32) prev[i] = -1;
+            __syncwarp();
+            for (int it = 0; it < 100 && !too_many; ++it) {
+                const int n0 = n;    // centres at the start of the round: cen; later ones: samples
+                auto centre = [&](int c) { return c < n0 ? cen + (size_t)c * K : X + (size_t)opened[c - n0] * K; };
+                auto beyond = [&](int i, int c, float d) -> int {   // FP64 distance > lambda
+                    if (FAST && fabsf(d - lamf) > slack(d) + 0x1p-22f * lamf) return d > lamf;
+                    return sqdist(X + (size_t)i * K, centre(c), K) > p.lambda;
+                };
+                // nearest existing centre of every sample (lowest index on ties)
+                for (int i = lane; i < S; i += 32) {
+                    int b = 0;
+                    float d1 = INFINITY, d2 = INFINITY;   // smallest and second smallest
+                    for (int c = 0; FAST && c < n0; ++c) {
+                        const float d = sqdist32(Xf + (size_t)i * K, cenf + (size_t)c * K, K);
+                        if (d < d1) {
+                            d2 = d1;
+                            d1 = d;
+                            b = c;
+                        } else {
+                            d2 = fminf(d2, d);
+                        }
+                    }
+                    // a NaN distance never compares smaller: the FP64 procedure decides
+                    if (!FAST || (n0 > 1 && !(d2 - d1 > slack(d1) + slack(d2))) || !(d1 < INFINITY)) {
+                        double db = INFINITY;
+                        b = 0;
+                        for (int c = 0; c < n0; ++c) {
+                            const double d = sqdist(X + (size_t)i * K, cen + (size_t)c * K, K);
+                            if (d < db) {
+                                db = d;
+                                b = c;
+                            }
+                        }
+                        d1 = (float)db;
+                        far[i] = db > p.lambda;
+                    } else {
+                        far[i] = beyond(i, b, d1);
+                    }
+                    assign[i] = b;
+                    dbf[i] = d1;
+                }
+                __syncwarp();
+                // samples in order: the next one farther than lambda from every centre opens a
+                // cluster; the later samples then compare with the new centre too
+                int pos = 0;
+                while (pos < S) {
+                    int found = S;
+                    for (int base = pos; base < S && found == S; base += 32) {
+                        const int i = base + lane;
+                        const unsigned v = __ballot_sync(kAll, i < S && far[i] != 0);
+                        if (v) found = base + __ffs(v) - 1;
+                    }
+                    if (found == S) break;
+                    if (n >= cap) {
+                        too_many = true;
+                        break;
+                    }
+                    const int c = n++;
+                    if (lane == 0) {
+                        opened[c - n0] = found;
+                        assign[found] = c;
+                    }
+                    __syncwarp();
+                    for (int j = found + 1 + lane; j < S; j += 32) {
+                        float d = 0.f, o = 0.f;
+                        if constexpr (FAST) d = sqdist32(Xf + (size_t)j * K, Xf + (size_t)found * K, K), o = dbf[j];
+                        bool nearer = d < o;
+                        if (!FAST || !(fabsf(d - o) > slack(d) + slack(o)))
+                            nearer = sqdist(X + (size_t)j * K, X + (size_t)found * K, K) <
+                                     sqdist(X + (size_t)j * K, centre(assign[j]), K);
+                        if (nearer) {
+                            dbf[j] = d;
+                            assign[j] = c;
+                            far[j] = beyond(j, c, d);
+                        }
+                    }
+                    __syncwarp();
+                    pos = found + 1;
+                }
+                if (too_many) break;
+                for (int c = lane; c < n; c += 32) cnt[c] = 0;
+                __syncwarp();
+                for (int i = lane; i < S; i += 32) atomicAdd(&cnt[assign[i]], 1);
+                __syncwarp();
+                // empty clusters are dropped (renumbered in order); offsets of the member lists
+                int m = 0;
+                for (int c0 = 0; c0 < n; c0 += 32) {
+                    const int c = c0 + lane;
+                    const unsigned v = __ballot_sync(kAll, c < n && cnt[c] > 0);
+                    if (c < n) map[c] = cnt[c] > 0 ? m + __popc(v & ((1u << lane) - 1u)) : -1;
+                    m += __popc(v);
+                }
+                __syncwarp();
+                int changed = 0;
+                for (int i = lane; i < S; i += 32) {
+                    const int a = map[assign[i]];
+                    assign[i] = a;
+                    changed |= a != prev[i];
+                    prev[i] = a;
+                }
+                __syncwarp();
+                // counts move down to their new numbers (a warp of them at a time, in order)
+                for (int c0 = 0; c0 < n; c0 += 32) {
+                    const int c = c0 + lane;
+                    const int to = c < n ? map[c] : -1, v = c < n ? cnt[c] : 0;
+                    __syncwarp();
+                    if (to >= 0) cnt[to] = v;
+                    __syncwarp();
+                }
+                n = m;
+                if (lane == 0) {
+                    int s = 0;
+                    for (int c = 0; c < n; ++c) off[c] = s, s += cnt[c];
+                    off[n] = s;
+                }
+                __syncwarp();
+                for (int c = lane; c < n; c += 32) map[c] = off[c];   // next free place
+                __syncwarp();
+                for (int i0 = 0; i0 < S; i0 += 32) {
+                    const int i = i0 + lane;
+                    const int a = i < S ? assign[i] : -1;
+                    const unsigned same = __match_any_sync(kAll, a);
+                    const int rank = __popc(same & ((1u << lane) - 1u));
+                    const int at = a >= 0 ? map[a] : 0;
+                    __syncwarp();
+                    if (a >= 0) {
+                        member[at + rank] = i;
+                        if (rank == 0) map[a] = at + __popc(same);
+                    }
+                    __syncwarp();
+                }
+                // centres to the means of their samples, in order
+                for (int e = lane; e < n * K; e += 32) {
+                    const int c = e / K, k = e % K;
+                    double s = 0.0;
+                    for (int q = off[c]; q < off[c + 1]; ++q) s = dadd(s, X[(size_t)member[q] * K + k]);
+                    const double mean = s / (double)cnt[c];
+                    cen[e] = mean;
+                    if constexpr (FAST) cenf[e] = (float)mean;
+                }
+                __syncwarp();
+                if (!__any_sync(kAll, changed)) break;
+            }
+        }
+        if (too_many) {
+            if (lane == 0) over[atomicAdd(over_n, 1)] = (int32_t)row;
+            continue;
+        }
+        if (p.assign)
+            for (int i = lane; i < S; i += 32) p.assign[row * S + i] = p.mode != 0 ? assign[i] : 0;
+        // the chosen clusters, largest first (ties: lowest index), with at least K + 1 samples
+        const int64_t q = p.pi ? row : p.row0 + row;
+        int used = 0;
         if (p.mode != 0) {
             const int want = p.mode == 1 ? 1 : C;
             for (int t = 0; t < want; ++t) {
-                int b = -1;
-                for (int c = 0; c < n; ++c)
-                    if (sizes[c] >= 0 && (b < 0 || sizes[c] > sizes[b])) b = c;
-                if (b < 0) break;
-                const int sz = sizes[b];
-                sizes[b] = -1;
-                if (sz < K + 1) continue;
-                chosen[used] = b;
-                map[used] = sz;              // component size
+                int best = -1, size = -1;
+                for (int c = lane; c < n; c += 32)
+                    if (cnt[c] > size) size = cnt[c], best = c;
+                // the warp's largest (size, then lowest index) as one key
+                unsigned key = best < 0 ? 0u : (unsigned)size << 16 | (0xffffu - (unsigned)best);
+                key = __reduce_max_sync(kAll, key);
+                if (key == 0u) break;
+                best = 0xffff - (int)(key & 0xffffu);
+                size = (int)(key >> 16);
+                __syncwarp();
+                if (lane == 0) cnt[best] = -1;
+                __syncwarp();
+                if (size < K + 1) break;      // the remaining ones are no larger
+                if (lane == 0) map[used] = best;
                 ++used;
             }
         }
-        misc[1] = used;
-    }
-    __syncwarp();
-    used = misc[1];
-    // Gaussian of the samples of cluster cl (all samples when cl < 0): mean into m, precision
-    // (inverse of the 1/n covariance) into Lam; false when fewer than K + 1 samples or singular
-    auto fit = [&](int cl, double *m) -> bool {
-        int nn = 0;
-        for (int i = 0; i < S; ++i) nn += (cl < 0 || assign[i] == cl);
-        if (nn < K + 1) return false;
-        for (int k = lane; k < K; k += 32) {
-            double s = 0.0;
-            for (int i = 0; i < S; ++i)
-                if (cl < 0 || assign[i] == cl) s = dadd(s, X[(size_t)i * K + k]);
-            m[k] = s / (double)nn;
-        }
         __syncwarp();
-        for (int e = lane; e < K * K; e += 32) {
-            const int a = e / K, b = e % K;
-            double s = 0.0;
-            for (int i = 0; i < S; ++i)
-                if (cl < 0 || assign[i] == cl)
-                    s = dadd(s, dmul(dsub(X[(size_t)i * K + a], m[a]), dsub(X[(size_t)i * K + b], m[b])));
-            Sig[e] = s / (double)nn;
-        }
-        __syncwarp();
-        return warp_spd_inverse(Sig, Lam, Lw, col, K, lane);
-    };
-    double wts[kMaxComponents] = {0.0, 0.0, 0.0, 0.0};
-    int got = 0;
-    bool bad = false;
-    for (int t = 0; t < used; ++t) {
-        const int cl = chosen[t];
-        const int sz = map[t];
-        __syncwarp();
-        if (!fit(cl, fmu + (size_t)got * K)) continue;
-        // keep this component's precision for the outputs
-        for (int e = lane; e < K * K; e += 32) cL[(size_t)got * K * K + e] = Lam[e];
-        wts[got] = (double)sz;
-        ++got;
-    }
-    if (got == 0) {
-        // moment matching over all samples
-        __syncwarp();
-        if (!fit(-1, fmu)) {
-            bad = true;
-        } else {
-            for (int e = lane; e < K * K; e += 32) cL[e] = Lam[e];
-            wts[0] = 1.0;
-            got = 1;
-        }
-    }
-    if (bad) {
-        if (lane == 0) {
-            atomicOr(&p.err->flags, ERR_NOT_PD);
-            atomicMin(&p.err->first_bad_row, (int)(p.row0 + row));
-        }
-        return;
-    }
-    double tot = 0.0;
-    for (int c = 0; c < got; ++c) tot = dadd(tot, wts[c]);
-    for (int c = 0; c < got; ++c) wts[c] = wts[c] / tot;
-    __syncwarp();
-    // pooled mean and covariance: sum_c pi_c (Lambda_c^{-1} + (mu_c - m)(mu_c - m)^T)
-    for (int k = lane; k < K; k += 32) {
-        double s = 0.0;
-        for (int c = 0; c < got; ++c) s = dadd(s, dmul(wts[c], fmu[(size_t)c * K + k]));
-        pm[k] = s;
-    }
-    for (int e = lane; e < K * K; e += 32) Acc[e] = 0.0;
-    __syncwarp();
-    for (int c = 0; c < got; ++c) {
-        const double *Lc = cL + (size_t)c * K * K;
-        for (int e = lane; e < K * K; e += 32) Sig[e] = Lc[e];
-        __syncwarp();
-        if (!warp_spd_inverse(Sig, Lam, Lw, col, K, lane)) {
-            bad = true;
-            break;
-        }
-        const double *mc = fmu + (size_t)c * K;
-        for (int e = lane; e < K * K; e += 32) {
-            const int a = e / K, b = e % K;
-            Acc[e] = dadd(Acc[e], dmul(wts[c], dadd(Lam[e], dmul(dsub(mc[a], pm[a]), dsub(mc[b], pm[b])))));
-        }
-        __syncwarp();
-    }
-    if (!bad) bad = !warp_spd_inverse(Acc, Sig, Lw, col, K, lane);   // pooled precision in Sig
-    if (bad) {
-        if (lane == 0) {
-            atomicOr(&p.err->flags, ERR_NOT_PD);
-            atomicMin(&p.err->first_bad_row, (int)(p.row0 + row));
-        }
-        return;
-    }
-    // ---- outputs --------------------------------------------------------------------------
-    const int64_t KK = (int64_t)K * K;
-    if (p.pi) {
-        for (int c = lane; c < C; c += 32) p.pi[row * C + c] = c < got ? wts[c] : 0.0;
-        for (int e = lane; e < C * K; e += 32) {
-            const int c = e / K;
-            p.mu[row * C * K + e] = c < got ? fmu[e] : 0.0;
-        }
-        for (int64_t e = lane; e < C * KK; e += 32) {
-            const int c = (int)(e / KK);
-            p.Lam[row * C * KK + e] = c < got ? cL[(size_t)c * KK + (e % KK)] : 0.0;
-        }
-        for (int k = lane; k < K; k += 32) p.pooled_mu[row * K + k] = pm[k];
-        for (int e = lane; e < KK; e += 32) p.pooled_Lam[row * KK + e] = Sig[e];
-    }
-    if (p.mm_mu) {
-        // the summary the library propagates and aggregates: the dominant component (mode 1)
-        // or the pooled moments (mode 2), as mean, packed precision and precision x mean
-        const int64_t ar = p.row0 + row;
-        const double *sm = p.mode == 1 ? fmu : pm;
-        const double *sL = p.mode == 1 ? cL : Sig;
-        for (int k = lane; k < K; k += 32) p.mm_mu[ar * K + k] = sm[k];
-        for (int e = lane; e < K * (K + 1) / 2; e += 32) {
-            int i = 0;
-            while ((i + 1) * (i + 2) / 2 <= e) ++i;
-            const int j = e - i * (i + 1) / 2;
-            p.mm_L[(int64_t)e * p.R + ar] = sL[i * K + j];
-        }
-        for (int i = lane; i < K; i += 32) {
-            double acc = 0.0;
-            for (int k = 0; k < K; ++k) acc = fma(sL[i * K + k], sm[k], acc);
-            p.mm_b[(int64_t)i * p.R + ar] = acc;
-        }
-        if (p.mix) {
-            // mixture store of the row: per component [log pi + log det(Lambda)/2][mu][L packed]
-            // [Lambda mu]; unused components get a -infinity score
-            const int NT = K * (K + 1) / 2, W = 1 + 2 * K + NT;
-            double *mx = p.mix + ar * (int64_t)C * W;
-            for (int c = 0; c < C; ++c) {
-                double *o = mx + (int64_t)c * W;
-                if (c >= got) {
-                    if (lane == 0) o[0] = -INFINITY;
-                    continue;
-                }
-                const double *Lc = cL + (size_t)c * KK;
-                const double *mc = fmu + (size_t)c * K;
-                __syncwarp();
-                const bool okc = warp_chol(Lc, Lw, K, lane);
-                if (lane == 0) {
-                    double logdet = 0.0;
-                    for (int k = 0; k < K; ++k) logdet += 2.0 * log(Lw[k * K + k]);
-                    o[0] = okc ? log(wts[c]) + 0.5 * logdet : -INFINITY;
-                }
-                for (int k = lane; k < K; k += 32) o[1 + k] = mc[k];
-                for (int e = lane; e < NT; e += 32) {
-                    int i = 0;
-                    while ((i + 1) * (i + 2) / 2 <= e) ++i;
-                    const int j = e - i * (i + 1) / 2;
-                    o[1 + K + e] = Lc[i * K + j];
-                }
-                for (int i = lane; i < K; i += 32) {
-                    double acc = 0.0;
-                    for (int k = 0; k < K; ++k) acc = fma(Lc[i * K + k], mc[k], acc);
-                    o[1 + K + NT + i] = acc;
-                }
+        // centred members in place, then the packed covariances of all chosen clusters
+        for (int t = 0; t < used; ++t) {
+            const int c = map[t], b0 = off[c], m = off[c + 1] - b0;
+            for (int e = lane; e < m * K; e += 32) {
+                const int k = e % K;
+                X[(size_t)member[b0 + e / K] * K + k] -= cen[(size_t)c * K + k];
             }
+            for (int k = lane; k < K; k += 32) fs.mean(q, t, k) = cen[(size_t)c * K + k];
+            if (lane == 0) fs.size(q, t) = (double)m;
+        }
+        if (lane == 0 && used < C) fs.size(q, used) = 0.0;
+        __syncwarp();
+        for (int e = lane; e < used * NT; e += 32) {
+            const int t = e / NT, c = map[t];
+            int i = 0, j = e % NT;
+            while (j > i) j -= ++i;
+            double s = 0.0;
+            for (int b = off[c]; b < off[c + 1]; ++b) {
+                const double *x = X + (size_t)member[b] * K;
+                s = fma(x[i], x[j], s);
+            }
+            fs.cov(q, t, e % NT) = s / (double)(off[c + 1] - off[c]);
         }
     }
 }
 
-void launch_summary(const SummaryParams &p, cudaStream_t st)
+// The rows' precisions from their covariances, one thread per row (FP64 warp instructions cost the
+// same whatever their active lanes: a warp per row spent 32 times the instructions, and its
+// serial Cholesky and divisions their latency): component precisions (a component with a singular
+// covariance is dropped; a row without one takes all its samples), the mixture's pooled mean and
+// covariance sum_c pi_c (Sigma_c + (mu_c - m)(mu_c - m)^T), its precision, and the outputs.
+__global__ void __launch_bounds__(kRowBlock) fit_kernel(SummaryParams p)
 {
-    if (p.n_rows <= 0) return;
-    const size_t smem = summary_smem(p.K, p.S);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(summary_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    summary_kernel<<<(unsigned)p.n_rows, 32, smem, st>>>(p);
+    extern __shared__ double sh[];
+    const int t = threadIdx.x, rb = blockDim.x;
+    const int64_t row = (int64_t)blockIdx.x * rb + t;
+    if (row >= p.n_rows) return;
+    const int K = p.K, S = p.S, C = p.C, NT = ntri(K);
+    const int64_t q = p.pi ? row : p.row0 + row, KK = (int64_t)K * K, W = 1 + 2 * K + NT;
+    const FitStage fs = fit_stage(p);
+    double *A = sh + t, *Acc = A + NT * rb, *v = Acc + NT * rb, *pm = v + K * rb;
+    auto bad_row = [&]() {
+        atomicOr(&p.err->flags, ERR_NOT_PD);
+        atomicMin(&p.err->first_bad_row, (int)(p.row0 + row));
+    };
+    // component c's precision (packed in A) to its place
+    auto keep_component = [&](int c, double logdet) {
+        if (p.pi) {
+            for (int i = 0; i < K; ++i)
+                for (int j = 0; j <= i; ++j) {
+                    const double l = RS(A, tri(i, j));
+                    p.Lam[(q * C + c) * KK + i * K + j] = l;
+                    p.Lam[(q * C + c) * KK + j * K + i] = l;
+                }
+        } else if (p.mix) {
+            double *o = p.mix + (q * C + c) * W;
+            o[0] = logdet;    // + log pi once the weights are known
+            for (int e = 0; e < NT; ++e) o[1 + K + e] = RS(A, e);
+            for (int i = 0; i < K; ++i) {
+                double s = 0.0;
+                for (int k = 0; k < K; ++k)
+                    s = fma(RS(A, i >= k ? tri(i, k) : tri(k, i)), o[1 + k], s);
+                o[1 + K + NT + i] = s;
+            }
+        }
+    };
+    double w[kMaxComponents] = {0.0, 0.0, 0.0, 0.0};
+    // components whose precision exists add their covariance to the pooled one in Acc
+    double tot = 0.0;
+    int got = 0;
+    for (int e = 0; e < NT; ++e) RS(Acc, e) = 0.0;
+    auto add = [&](int src, int dst, double size) -> bool {
+        for (int e = 0; e < NT; ++e) RS(A, e) = fs.cov(q, src, e);
+        double logdet = 0.0;
+        if (!row_spd_inverse(A, v, K, rb, p.mix ? &logdet : nullptr)) return false;
+        for (int e = 0; e < NT; ++e) RS(Acc, e) = fma(size, fs.cov(q, src, e), RS(Acc, e));
+        if (dst != src)
+            for (int k = 0; k < K; ++k) fs.mean(q, dst, k) = fs.mean(q, src, k);
+        keep_component(dst, logdet);
+        w[dst] = size;
+        tot += size;
+        return true;
+    };
+    for (int c = 0; c < C && p.mode != 0; ++c) {
+        const double size = fs.size(q, c);
+        if (!(size > 0.0)) break;
+        if (add(c, got, size)) ++got;
+    }
+    if (got == 0) {
+        // moment matching over all samples
+        bool ok = S >= K + 1;
+        if (ok) {
+            const double *x = p.samples + (p.row0 + row) * K;
+            for (int k = 0; k < K; ++k) {
+                double s = 0.0;
+                for (int i = 0; i < S; ++i) s = dadd(s, x[(int64_t)i * p.sample_stride + k]);
+                fs.mean(q, 0, k) = s / (double)S;
+            }
+            for (int e = 0; e < NT; ++e) RS(A, e) = 0.0;
+            for (int i = 0; i < S; ++i) {
+                for (int k = 0; k < K; ++k) RS(v, k) = x[(int64_t)i * p.sample_stride + k] - fs.mean(q, 0, k);
+                for (int a = 0; a < K; ++a)
+                    for (int b = 0; b <= a; ++b) RS(A, tri(a, b)) = fma(RS(v, a), RS(v, b), RS(A, tri(a, b)));
+            }
+            for (int e = 0; e < NT; ++e) fs.cov(q, 0, e) = RS(A, e) / (double)S;
+            ok = add(0, 0, 1.0);
+        }
+        if (!ok) {
+            bad_row();
+            return;
+        }
+        got = 1;
+    }
+    // pooled mean, and the components' spread about it
+    for (int i = 0; i < K; ++i) {
+        double s = 0.0;
+        for (int c = 0; c < got; ++c) s = fma(w[c] / tot, fs.mean(q, c, i), s);
+        RS(pm, i) = s;
+    }
+    for (int c = 0; c < got; ++c) {
+        for (int i = 0; i < K; ++i) RS(v, i) = fs.mean(q, c, i) - RS(pm, i);
+        for (int i = 0; i < K; ++i) {
+            const double wi = w[c] * RS(v, i);
+            for (int j = 0; j <= i; ++j) RS(Acc, tri(i, j)) = fma(wi, RS(v, j), RS(Acc, tri(i, j)));
+        }
+    }
+    const double inv = 1.0 / tot;
+    for (int e = 0; e < NT; ++e) RS(A, e) = RS(Acc, e) * inv;
+    if (!row_spd_inverse(A, v, K, rb, nullptr)) {
+        bad_row();
+        return;
+    }
+    if (p.pi) {
+        for (int c = 0; c < C; ++c) {
+            p.pi[q * C + c] = c < got ? w[c] / tot : 0.0;
+            for (int k = 0; k < K && c >= got; ++k) p.mu[(q * C + c) * K + k] = 0.0;
+            for (int64_t e = 0; e < KK && c >= got; ++e) p.Lam[(q * C + c) * KK + e] = 0.0;
+        }
+        for (int i = 0; i < K; ++i) {
+            p.pooled_mu[q * K + i] = RS(pm, i);
+            for (int j = 0; j <= i; ++j) {
+                p.pooled_Lam[q * KK + i * K + j] = RS(A, tri(i, j));
+                p.pooled_Lam[q * KK + j * K + i] = RS(A, tri(i, j));
+            }
+        }
+    }
+    if (p.mm_mu) {
+        // the summary the library propagates and aggregates: the dominant component (mode 1:
+        // one component, so its pooled moments are its own) or the pooled moments, as mean,
+        // packed precision and precision x mean
+        for (int k = 0; k < K; ++k) p.mm_mu[q * K + k] = RS(pm, k);
+        for (int e = 0; e < NT; ++e) p.mm_L[(int64_t)e * p.R + q] = RS(A, e);
+        for (int i = 0; i < K; ++i) {
+            double s = 0.0;
+            for (int k = 0; k < K; ++k) s = fma(RS(A, i >= k ? tri(i, k) : tri(k, i)), RS(pm, k), s);
+            p.mm_b[(int64_t)i * p.R + q] = s;
+        }
+        // mixture store: [log pi + log det(Lambda)/2][mu][L packed][Lambda mu]; unused
+        // components get a -infinity score
+        for (int c = 0; p.mix && c < C; ++c) {
+            double &score = p.mix[(q * C + c) * W];
+            score = c < got ? log(w[c] / tot) + score : -INFINITY;
+        }
+    }
+}
+
+cudaError_t launch_summary(const SummaryParams &p, cudaStream_t st)
+{
+    if (p.n_rows <= 0) return cudaSuccess;
+    // first launch: a warp per row with room for kFastCentres clusters; second: the listed rows
+    const int cap = kFastCentres, all = 2 * p.S + 1;
+    const size_t smem = cluster_smem(p.K, p.S, cap, true), smem_all = cluster_smem(p.K, p.S, all, false);
+    cudaError_t e = cudaSuccess;
+    // samples too many for the FP32 copies to fit beside them: every row takes the second form
+    const bool fast = smem <= 200 * 1024;
+    if (fast && smem > 48 * 1024)
+        e = cudaFuncSetAttribute(cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && smem_all > 48 * 1024)
+        e = cudaFuncSetAttribute(cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_all);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p.over_n, 0, sizeof(int32_t), st);
+    if (e != cudaSuccess) return e;
+    if (fast)
+        cluster_kernel<true><<<(unsigned)p.n_rows, 32, smem, st>>>(p, cap, nullptr, nullptr, p.over, p.over_n);
+    if (!fast || p.mode != 0)
+        cluster_kernel<false><<<(unsigned)std::min<int64_t>(p.n_rows, fast ? 304 : p.n_rows), 32, smem_all, st>>>(
+            p, all, fast ? p.over : nullptr, fast ? p.over_n : nullptr, nullptr, nullptr);
+    const size_t per = 2 * (size_t)ntri(p.K) + 2 * p.K;
+    const int rb = row_block(per);
+    const size_t fit = per * rb * sizeof(double);
+    if (fit > 48 * 1024)
+        e = cudaFuncSetAttribute(fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fit);
+    if (e != cudaSuccess) return e;
+    fit_kernel<<<(unsigned)((p.n_rows + rb - 1) / rb), rb, fit, st>>>(p);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------

@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 def _reference(seed, t, tag, n):
-    b = np.random.Philox(key=[seed, 0])
+    b = np.random.Philox(key=np.array([seed, 0], np.uint64))
     start = (t << 64) + (tag << 128) - 1          # numpy steps the counter before each call
     st = b.state
     st["state"]["counter"] = np.array([(start >> (64 * k)) & (2 ** 64 - 1) for k in range(4)], np.uint64)
