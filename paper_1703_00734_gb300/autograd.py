@@ -25,11 +25,10 @@ class LogJoint(torch.autograd.Function):
                                           float(log_alpha), gX.data_ptr(), gW.data_ptr())
         fctx.save_for_backward(gX, gW)
         fctx.g_la = g_la
-        return torch.tensor(value, dtype=torch.float64, device=X.device)
+        return X.new_full((), value, dtype=torch.float64)
 
     @staticmethod
     def backward(fctx, g):
         gX, gW = fctx.saved_tensors
         gf = g.to(torch.float32)
-        g_la = torch.as_tensor(fctx.g_la, dtype=torch.float64, device=g.device) * g
-        return None, None, gX * gf, gW * gf, g_la
+        return None, None, gX * gf, gW * gf, fctx.g_la * g

@@ -2414,12 +2414,13 @@ bmf_status grow(bmf_ctx *c, T *&p, int64_t &cap, int64_t need)
 }
 
 struct LogJoint {
-    double r2 = 0.0, quad = 0.0, value = 0.0, g_log_alpha = 0.0;
+    double value = 0.0, g_log_alpha = 0.0;
 };
 
-// Gradient of the subset's log-joint at (X, W) into (gX, gW); scalar parts on the host.
+// Gradient of the subset's log-joint at (X, W) into (gX, gW), enqueued; with `out` the scalar parts
+// are read back, which waits for them.
 bmf_status logjoint(bmf_ctx *c, int32_t subset, const float *X, const float *W, int64_t ld,
-                    double log_alpha, float *gX, float *gW, LogJoint &out)
+                    double log_alpha, float *gX, float *gW, LogJoint *out)
 {
     const SubsetGeom &g = c->P.subs[subset];
     const int K = c->K, kt = adjoint_kt(K), ldp = adjoint_ld(K);
@@ -2429,10 +2430,10 @@ bmf_status logjoint(bmf_ctx *c, int32_t subset, const float *X, const float *W, 
         const Side &me = f == 0 ? c->X : c->W;
         const int64_t r0 = f == 0 ? g.xoff : g.woff, r1 = r0 + (f == 0 ? g.n() : g.d());
         need_part = std::max(need_part, (me.h_item_ptr[r1] - me.h_item_ptr[r0]) * ldp);
-        nb[f] = adjoint_row_blocks(r1 - r0);
+        nb[f] = adjoint_row_blocks(r1 - r0, kt, c->sms);
     }
     bmf_status s = grow(c, c->adj_part, c->adj_part_cap, need_part);
-    if (!s) s = grow(c, c->adj_sums, c->adj_sums_cap, 2 * (nb[0] + nb[1]));
+    if (!s) s = grow(c, c->adj_sums, c->adj_sums_cap, 2 * (nb[0] + nb[1]) + 2);
     if (s) return s;
     for (int f = 0; f < 2 && c->prec == BMF_FP64; ++f)
         if (!c->fval[f]) {
@@ -2470,22 +2471,21 @@ bmf_status logjoint(bmf_ctx *c, int32_t subset, const float *X, const float *W, 
         ap.grad = f == 0 ? gX : gW;
         ap.alpha = alpha;
         ap.count_r2 = f == 0 ? 1 : 0;
+        ap.row_blocks = (int)nb[f];
         ap.block_sums = c->adj_sums + (f == 0 ? 0 : 2 * nb[0]);
         traced(c, c->st, K_ADJ, 2, [&] { launch_adjoint(ap, c->sms * 8, c->st); });
     }
     CUDA_TRY(c, cudaGetLastError());
-    std::vector<double> h(2 * (nb[0] + nb[1]));
-    CUDA_TRY(c, cudaMemcpyAsync(h.data(), c->adj_sums, h.size() * sizeof(double),
-                                cudaMemcpyDeviceToHost, c->st));
+    if (!out) return BMF_OK;
+    double *sums = c->adj_sums + 2 * (nb[0] + nb[1]);
+    launch_adjoint_sums(c->adj_sums, (int)(nb[0] + nb[1]), sums, c->st);
+    CUDA_TRY(c, cudaMemcpyAsync(c->rb->rmse, sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CUDA_TRY(c, cudaStreamSynchronize(c->st));
-    out.r2 = out.quad = 0.0;
-    for (int64_t b = 0; b < nb[0] + nb[1]; ++b) {
-        out.r2 += h[2 * b];
-        out.quad += h[2 * b + 1];
-    }
+    ++c->launches;
+    const double r2 = c->rb->rmse[0], quad = c->rb->rmse[1];
     const double M = (double)g.nnz;
-    out.value = -0.5 * alpha * out.r2 + 0.5 * M * log_alpha - 0.5 * out.quad;
-    out.g_log_alpha = 0.5 * M - 0.5 * alpha * out.r2;
+    out->value = -0.5 * alpha * r2 + 0.5 * M * log_alpha - 0.5 * quad;
+    out->g_log_alpha = 0.5 * M - 0.5 * alpha * r2;
     return BMF_OK;
 }
 
@@ -2529,7 +2529,7 @@ bmf_status bmf_logjoint_grad(bmf_ctx *c, int32_t subset, const float *X, const f
         return fail(c, BMF_E_ARG, "factors must be 16-byte aligned with ld >= K and ld % 4 == 0");
     if (!std::isfinite(log_alpha)) return fail(c, BMF_E_NONFINITE, "non-finite log_alpha");
     LogJoint lj;
-    bmf_status s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, lj);
+    bmf_status s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, &lj);
     if (s) return s;
     if (c->prof) collect_profile(c);
     if (value) *value = lj.value;
@@ -2550,42 +2550,56 @@ bmf_status bmf_langevin(bmf_ctx *c, int32_t subset, int32_t n_steps, float *X, f
     const SubsetGeom &g = c->P.subs[subset];
     const int64_t n = g.n(), d = g.d(), K = c->K;
     const int64_t sx = n * ld, sw = d * ld;
+    if (!uniforms) {
+        // every proposal is taken: the moves and gradients follow one another on the stream, in
+        // place, and only the final value is read back
+        bmf_status s = grow(c, c->lg_buf, c->lg_cap, sx + sw + 8);
+        if (s) return s;
+        float *gX = c->lg_buf, *gW = gX + sx;
+        LogJoint last;
+        s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, n_steps == 0 ? &last : nullptr);
+        for (int32_t it = 0; it < n_steps && !s; ++it) {
+            const float *xi = noise + (int64_t)it * (n + d) * K;
+            traced(c, c->st, K_ADJ, 1, [&] {
+                launch_langevin(X, W, gX, gW, X, W, xi, n, d, (int)K, (int)ld, (float)eps, c->st);
+            });
+            s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, it + 1 == n_steps ? &last : nullptr);
+        }
+        if (s) return s;
+        if (c->prof) collect_profile(c);
+        if (accepted) *accepted = n_steps;
+        if (value) *value = last.value;
+        return BMF_OK;
+    }
     // buffers: gradient at the current state (gX, gW), proposal (pX, pW), its gradient (qX, qW)
     bmf_status s = grow(c, c->lg_buf, c->lg_cap, 3 * (sx + sw) + 8);
     if (s) return s;
     float *gX = c->lg_buf, *gW = gX + sx, *pX = gW + sw, *pW = pX + sx, *qX = pW + sw, *qW = qX + sx;
     LogJoint cur, prop;
-    s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, cur);
+    s = logjoint(c, subset, X, W, ld, log_alpha, gX, gW, &cur);
     if (s) return s;
     int32_t acc = 0;
     for (int32_t it = 0; it < n_steps; ++it) {
         const float *xi = noise + (int64_t)it * (n + d) * K;
-        CUDA_TRY(c, cudaMemcpyAsync(pX, X, sx * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-        CUDA_TRY(c, cudaMemcpyAsync(pW, W, sw * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-        traced(c, c->st, K_ADJ, 2, [&] {
-            launch_langevin(pX, gX, xi, n, (int)K, (int)ld, (float)eps, c->st);
-            launch_langevin(pW, gW, xi + n * K, d, (int)K, (int)ld, (float)eps, c->st);
+        traced(c, c->st, K_ADJ, 1, [&] {
+            launch_langevin(X, W, gX, gW, pX, pW, xi, n, d, (int)K, (int)ld, (float)eps, c->st);
         });
-        s = logjoint(c, subset, pX, pW, ld, log_alpha, qX, qW, prop);
+        s = logjoint(c, subset, pX, pW, ld, log_alpha, qX, qW, &prop);
         if (s) return s;
-        bool take = true;
-        if (uniforms) {
-            // log A = l' - l + log q(theta | theta') - log q(theta' | theta),
-            // log q(a | b) = -|a - b - (eps/2) grad l(b)|^2 / (2 eps)
-            bmf_status e1, e2, e3, e4;
-            const double back = sqdiff(c, X, pX, qX, 0.5 * eps, n, ld, e1) +
-                                sqdiff(c, W, pW, qW, 0.5 * eps, d, ld, e2);
-            const double fwd = sqdiff(c, pX, X, gX, 0.5 * eps, n, ld, e3) +
-                               sqdiff(c, pW, W, gW, 0.5 * eps, d, ld, e4);
-            if (e1 || e2 || e3 || e4) return BMF_E_CUDA;
-            const double logA = prop.value - cur.value - back / (2 * eps) + fwd / (2 * eps);
-            take = std::log(uniforms[it]) < logA;
-        }
-        if (take) {
+        // log A = l' - l + log q(theta | theta') - log q(theta' | theta),
+        // log q(a | b) = -|a - b - (eps/2) grad l(b)|^2 / (2 eps)
+        bmf_status e1, e2, e3, e4;
+        const double back = sqdiff(c, X, pX, qX, 0.5 * eps, n, ld, e1) +
+                            sqdiff(c, W, pW, qW, 0.5 * eps, d, ld, e2);
+        const double fwd = sqdiff(c, pX, X, gX, 0.5 * eps, n, ld, e3) +
+                           sqdiff(c, pW, W, gW, 0.5 * eps, d, ld, e4);
+        if (e1 || e2 || e3 || e4) return BMF_E_CUDA;
+        const double logA = prop.value - cur.value - back / (2 * eps) + fwd / (2 * eps);
+        if (std::log(uniforms[it]) < logA) {
             CUDA_TRY(c, cudaMemcpyAsync(X, pX, sx * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
             CUDA_TRY(c, cudaMemcpyAsync(W, pW, sw * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-            CUDA_TRY(c, cudaMemcpyAsync(gX, qX, sx * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-            CUDA_TRY(c, cudaMemcpyAsync(gW, qW, sw * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
+            std::swap(gX, qX);
+            std::swap(gW, qW);
             cur = prop;
             ++acc;
         }

@@ -290,7 +290,7 @@ bool launch_cond_pair(const CondParams &a, int n_blocks, cudaStream_t st);
 // Adjoint of the masked log-joint (adjoint.cu).
 int adjoint_kt(int K);          // template width (K rounded up to 4, 8, 12, 16, 32 or 64)
 int adjoint_ld(int K);          // floats per item partial
-int adjoint_row_blocks(int64_t n_rows);
+int adjoint_row_blocks(int64_t n_rows, int kt, int sms);
 struct AdjointParams {
     int K, kt, ldp;
     // pass 1: items items[0 .. n_items) (absolute index item_base + i)
@@ -311,11 +311,14 @@ struct AdjointParams {
     float *grad;                // [n_rows x ld]
     double alpha;
     int count_r2;
-    double *block_sums;         // [row blocks x 2]: sum r^2, sum prior quadratic
+    int row_blocks;             // grid of pass 2 (adjoint_row_blocks)
+    double *block_sums;         // [row blocks x 2]: sum r^2 (count_r2), sum prior quadratic
 };
 void launch_adjoint(const AdjointParams &a, int grid, cudaStream_t st);
-void launch_langevin(float *theta, const float *grad, const float *xi, int64_t n_rows, int K,
-                     int ld, float eps, cudaStream_t st);
+// out[0], out[1] = the sums of n block pairs.
+void launch_adjoint_sums(const double *sums, int n, double *out, cudaStream_t st);
+void launch_langevin(const float *X, const float *W, const float *gX, const float *gW, float *oX, float *oW,
+                     const float *xi, int64_t n_x, int64_t n_w, int K, int ld, float eps, cudaStream_t st);
 void launch_to_float(const double *in, float *out, int64_t n, cudaStream_t st);
 void launch_sqdiff(const float *a, const float *b, const float *g, double coef, int64_t n_rows,
                    int K, int64_t ld, double *block_sums, int blocks, cudaStream_t st);
