@@ -1704,7 +1704,10 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     c->rmse_part = c->mem.alloc<double>(2 * c->rmse_blocks);
     c->rmse_out = c->mem.alloc<double>(2);
     c->err_d = c->mem.alloc<DevError>(1);
-    c->gen_tab = c->mem.alloc<GenTables>(1);
+    // the normals' tables, except where reduced-precision gathers meet K > kPairsMaxK: rounding the
+    // draws differently there moves a chain by half of what its FP32 gathers are off by (see
+    // cond_pairs.cu), so they keep the FP64 functions
+    if (c->prec == BMF_FP64 || K <= kPairsMaxK) c->gen_tab = c->mem.alloc<GenTables>(1);
     c->aggX = c->mem.alloc<double>(N * K);
     c->aggW = c->mem.alloc<double>(D * K);
     c->ncorr_d = c->mem.alloc<unsigned long long>(1);
@@ -1761,7 +1764,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     }
     DevError z = {0u, INT32_MAX};
     cudaMemcpy(c->err_d, &z, sizeof(z), cudaMemcpyHostToDevice);
-    cudaMemcpy(c->gen_tab, &gen_tables(), sizeof(GenTables), cudaMemcpyHostToDevice);
+    if (c->gen_tab) cudaMemcpy(c->gen_tab, &gen_tables(), sizeof(GenTables), cudaMemcpyHostToDevice);
     // aggregation bases: X block i over submodels (i, j), then W block j over (i, j)
     {
         std::vector<int64_t> base((size_t)(I + J) * MB, 0);

@@ -344,7 +344,7 @@ struct GenParams {
     double *out;
     const int64_t *cnt_ptr;   // kind 4: W arena observation offsets (entries of a column)
     DevError *err;
-    const GenTables *tab;     // device copy of gen_tables()
+    const GenTables *tab;     // device copy of gen_tables(), or null for the FP64 functions
 };
 struct GenSubset {
     int32_t sid;

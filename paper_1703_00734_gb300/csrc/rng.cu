@@ -89,8 +89,23 @@ __device__ __forceinline__ double sqrt_unit(double t)
     return hi == 0 ? 0.0 : s;
 }
 
+// The same with the FP64 functions (rounded differently in the last bit).
+__device__ __forceinline__ void box_muller_fp64(uint64_t a, uint64_t b, double &z0, double &z1)
+{
+    const double r = sqrt(-2.0 * log(u_open0(a)));
+    double s, c;
+    sincos(6.283185307179586 * ((double)(b >> 11) * 0x1.0p-53), &s, &c);
+    z0 = r * c;
+    z1 = r * s;
+}
+
+template <bool TABLES>
 __device__ __forceinline__ void box_muller(uint64_t a, uint64_t b, const GenTables *tab, double &z0, double &z1)
 {
+    if constexpr (!TABLES) {
+        box_muller_fp64(a, b, z0, z1);
+        return;
+    }
     const double ln = log_unit((a >> 11) + 1, tab);
     // -2 ln u1 >= 0 (zero only for u1 = 1)
     const int lh = __double2hiint(ln) & 0x7fffffff;
@@ -119,6 +134,7 @@ __device__ __forceinline__ void box_muller(uint64_t a, uint64_t b, const GenTabl
     z1 = rad * __hiloint2double(__double2hiint(v) ^ nv, __double2loint(v));
 }
 
+template <bool TABLES>
 __global__ void __launch_bounds__(256) gen_kernel(GenParams p)
 {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -148,7 +164,7 @@ __global__ void __launch_bounds__(256) gen_kernel(GenParams p)
             uint64_t w[4] = {(uint64_t)l, (uint64_t)p.t, sg.tag, (uint64_t)j};
             philox4x64_10(w, p.seed, 0);
             double x, unused;
-            box_muller(w[0], w[1], p.tab, x, unused);
+            box_muller<TABLES>(w[0], w[1], p.tab, x, unused);
             double v = 1.0 + c * x;
             if (!(v > 0.0)) continue;
             v = v * v * v;
@@ -169,8 +185,8 @@ __global__ void __launch_bounds__(256) gen_kernel(GenParams p)
     uint64_t w[4] = {(uint64_t)l, (uint64_t)p.t, sg.tag, 0};
     philox4x64_10(w, p.seed, 0);
     double z[4];
-    box_muller(w[0], w[1], p.tab, z[0], z[1]);
-    box_muller(w[2], w[3], p.tab, z[2], z[3]);
+    box_muller<TABLES>(w[0], w[1], p.tab, z[0], z[1]);
+    box_muller<TABLES>(w[2], w[3], p.tab, z[2], z[3]);
     const int64_t e0 = 4 * l;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
@@ -180,7 +196,11 @@ __global__ void __launch_bounds__(256) gen_kernel(GenParams p)
 void launch_gen(const GenParams &p, cudaStream_t st)
 {
     if (p.n_units <= 0) return;
-    gen_kernel<<<(unsigned)((p.n_units + 255) / 256), 256, 0, st>>>(p);
+    const unsigned grid = (unsigned)((p.n_units + 255) / 256);
+    if (p.tab)
+        gen_kernel<true><<<grid, 256, 0, st>>>(p);
+    else
+        gen_kernel<false><<<grid, 256, 0, st>>>(p);
 }
 
 // Host side: the segments of one sweep's draw buffer for a batch (layout of the public header).
