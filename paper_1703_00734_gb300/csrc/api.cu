@@ -146,6 +146,7 @@ struct bmf_ctx {
     double *hyper = nullptr;         // [2 * S slots]
     double *stats = nullptr;
     int64_t stats_cap = 0;           // chunks
+    int *parts_done = nullptr;       // [chunks] parts of a conditional block drawn so far (zero when idle)
     HyperJob *d_jobs = nullptr;
     HyperJob *d_jobs2 = nullptr;     // the same jobs over the first-level partials
     std::vector<HyperJob> jobs_up;   // the job list last uploaded (skip identical uploads)
@@ -1048,6 +1049,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             cp.S1 = me.S1;
             cp.S2 = me.S2;
             cp.stats = c->stats;
+            cp.parts_done = c->parts_done;
             cp.err = c->err_d;
             cp.obs_ptr = me.ptr;
             cp.obs_idx = me.idx;
@@ -1068,7 +1070,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
                     // two lanes per row: the register-resident kernel where it exists
                     if (team == 2 && launch_cond_pair(q, (int)(bb - ba), sx)) return;
                     if (team > 1)
-                        launch_cond_team(c->prec, q, (int)(bb - ba), team, sx);
+                        launch_cond_team(c->prec, q, (int)(bb - ba), team, c->sms, sx);
                     else
                         launch_cond(c->prec, q, (int)(bb - ba), sx);
                 });
@@ -1674,6 +1676,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     c->W.stat0 = (int64_t)c->X.h_blocks.size();
     c->stats_cap = (int64_t)(c->X.h_blocks.size() + c->W.h_blocks.size());
     c->stats = c->mem.alloc<double>(c->stats_cap * (K + ntri(K)));
+    c->parts_done = c->mem.alloc<int>(c->stats_cap);
     c->d_jobs = c->mem.alloc<HyperJob>(kHyperJobsMax);
     c->d_jobs2 = c->mem.alloc<HyperJob>(kHyperJobsMax);
     c->stats2 = c->mem.alloc<double>((size_t)2 * S * kStatParts * (K + ntri(K)));
@@ -1756,6 +1759,7 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     cudaMemcpy(c->mu0_d, c->mu0.data(), K * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->W0inv_d, c->W0inv.data(), (size_t)K * K * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemset(c->hyper, 0, (size_t)2 * S * hyper_slot_len(K) * sizeof(double));
+    cudaMemset(c->parts_done, 0, std::max<int64_t>(c->stats_cap, 1) * sizeof(int));
     if (nt) {
         cudaMemcpy(c->trow, c->P.trow.data(), nt * sizeof(int32_t), cudaMemcpyHostToDevice);
         cudaMemcpy(c->tcol, c->P.tcol.data(), nt * sizeof(int32_t), cudaMemcpyHostToDevice);

@@ -353,9 +353,10 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
     const CondBlock blk = a.blocks[blockIdx.x];
     const int64_t R = a.R;
     const unsigned tmask = T == 32 ? 0xffffffffu : ((1u << T) - 1u) << (lane & ~(T - 1));
-    for (int q0 = 0; q0 < blk.n; q0 += n_teams) {
+    const int rows = kCondBlock / gridDim.y, q_end = min(blk.n, (int)(blockIdx.y + 1) * rows);
+    for (int q0 = blockIdx.y * rows; q0 < q_end; q0 += n_teams) {
         const int q = q0 + tm;
-        const bool active = q < blk.n;
+        const bool active = q < q_end;
         const int64_t r = blk.row0 + (active ? q : 0);
         bool bad = false;
         // G, r and the prior (teams past the block's rows carry an identity)
@@ -492,18 +493,18 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
     // factor draws its hyperparameters: every row of a block shares its subset's prior), read back
     // from the state rows this block has just written, each entry over the rows in order
     if (a.stats == nullptr || a.row_hslot[blk.row0] < 0) return;
-    __syncthreads();
+    if (!last_part(a.parts_done, a.blk0 + blockIdx.x, gridDim.y)) return;
     const int NS = K + NT;
     const double *Xb = a.X + blk.row0 * K;
     double *out = a.stats + (a.blk0 + blockIdx.x) * (int64_t)NS;
     for (int e = threadIdx.x; e < NS; e += blockDim.x) {
         double s = 0.0;
         if (e < K) {
-            for (int qq = 0; qq < blk.n; ++qq) s += Xb[qq * K + e];
+            for (int qq = 0; qq < blk.n; ++qq) s += __ldcg(Xb + qq * K + e);
         } else {
             int i, j;
             decode_tri(e - K, i, j);
-            for (int qq = 0; qq < blk.n; ++qq) s = fma(Xb[qq * K + i], Xb[qq * K + j], s);
+            for (int qq = 0; qq < blk.n; ++qq) s = fma(__ldcg(Xb + qq * K + i), __ldcg(Xb + qq * K + j), s);
         }
         out[e] = s;
     }
@@ -512,22 +513,23 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
 template <int T, int RMAX, typename GT>
 static void launch_team_t(const CondParams &a, int n_blocks, int sms, cudaStream_t st)
 {
-    // Threads per block (64 rows): a launch that leaves SMs idle spreads a block's rows over as many
-    // warps as it can, up to a row per team at once; otherwise small blocks, which fill an SM evenly
-    // (K = 10, 10,677 rows: 63 us with 64 threads for all, 32 us with this rule)
+    // A launch whose conditional blocks fit on the GPU at once takes the widest CUDA blocks that do:
+    // the rows go over more warps, and the block's statistics over more threads (K = 10, 10,677
+    // rows: 63 us with 64 threads, 32 us with 256).  Larger launches take 64 threads, which fill an
+    // SM evenly, and the rows of a conditional block in as many parts as rounds of its teams, until
+    // the launch fills the GPU about eight times over (K = 16, 45,000 rows: 245 us as one part, 149
+    // us in parts; 225,000 rows: 660 and 609 us).
     auto bytes = [&](int th) { return (size_t)(th / T) * team_pairs(a.K) * sizeof(fpair); };
-    int threads = 64;
-    for (int th = 256; th > 64; th /= 2) {
-        const int per_sm = std::min<int>((int)(220 * 1024 / bytes(th)), 512 / th);
-        if (th / T <= kCondBlock && n_blocks <= sms * per_sm) {
-            threads = th;
-            break;
-        }
-    }
+    auto fit = [&](int th) { return (int)std::min<size_t>(512 / th, (size_t)220 * 1024 / bytes(th)); };
+    int threads = 256, parts = 1;
+    while (threads > 64 && (threads / T > kCondBlock || n_blocks > sms * fit(threads))) threads /= 2;
+    const int teams = threads / T;
+    if (threads == 64)
+        while (parts < kCondBlock / teams && (int64_t)n_blocks * parts < (int64_t)8 * sms * fit(threads)) parts *= 2;
     const size_t smem = bytes(threads);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(cond_pairs_kernel<T, RMAX, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cond_pairs_kernel<T, RMAX, GT><<<n_blocks, threads, smem, st>>>(a);
+    cond_pairs_kernel<T, RMAX, GT><<<dim3(n_blocks, parts), threads, smem, st>>>(a);
 }
 
 template <typename GT>

@@ -83,6 +83,9 @@ struct CondParams {
     double *S2;                  // SoA [ntri(K)][R]
     double *stats;               // per-block sums of x and x x^T of the new state
                                  // [blocks x (K + ntri(K))], at slot blk0 + blockIdx.x
+    int *parts_done;             // [blocks], zero between launches: a conditional block's rows may be
+                                 // split over several CUDA blocks (cond_parts), the last of which
+                                 // forms the block's statistics
     DevError *err;
     // rows marked kFusedRow in multi_idx form their own Gram sums from their observations (in
     // list order), which the Gram pass skips: the row's list and the gathered partner copy
@@ -106,6 +109,31 @@ bool launch_cond_pairs(int prec, const CondParams &a, int n_blocks, int sms, cud
 constexpr int32_t kFusedRow = -2;
 constexpr int kFuseMaxObs = 64;
 constexpr int kCondBlock = 64;
+
+// CUDA blocks (grid y) that share a conditional block's rows: part p of `parts` draws the rows
+// [p, p + 1) kCondBlock / parts.  A block of rows drawn a few at a time by one CUDA block leaves
+// SMs waiting for the last ones; parts of a round's rows each even that out.
+#ifdef __CUDACC__
+// Whether this CUDA block is the last of its conditional block's parts to finish: the others' rows
+// are then visible to it.  Called by all threads, after the part's rows are written.
+__device__ __forceinline__ bool last_part(int *parts_done, int64_t block, int parts)
+{
+    if (parts == 1) {
+        __syncthreads();
+        return true;
+    }
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(parts_done + block, 1) == parts - 1;
+        if (last) parts_done[block] = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
+}
+#endif
 
 // Per-chunk sums for the hyperparameter step: for each chunk, sum x and the packed lower
 // sum x x^T over rows [r0, r1) of an FP64 arena.
@@ -278,7 +306,7 @@ int wide_part_ld(int K);
 void launch_gram_wide(int K, int prec, const GramParams &a, int grid, cudaStream_t st,
                       bool tf32_single = false);
 // Conditional draw with a team of `team` lanes (4, 8, 16 or 32) per row (wide.cu).
-void launch_cond_team(int prec, const CondParams &a, int n_blocks, int team, cudaStream_t st);
+void launch_cond_team(int prec, const CondParams &a, int n_blocks, int team, int sms, cudaStream_t st);
 int cond_team_size(int K);
 // Whether the conditional can factor a row of dimension K with `lanes` lanes: two lanes (the
 // register-resident kernel) for 13 <= K <= 16, else a team whose rows fit in shared memory.
