@@ -349,8 +349,8 @@ bool host_inverse(int K, const std::vector<double> &A, std::vector<double> &Ainv
 const SubsetGeom &geom_of_slot(const bmf_ctx *c, int sl) { return c->P.subs[c->P.slot_sid[sl]]; }
 
 // Gram partial layout: entries per item and the offset of the right-hand side.
-int part_nv(int K) { return K > kNarrowMaxK ? ntri(K) + K : gram_nv(padded_k(K)); }
-int part_rhs_of(int K) { return K > kNarrowMaxK ? ntri(K) : ntri(padded_k(K)); }
+int part_nv(int K, int prec) { return gram_nv(K > kNarrowMaxK ? K : gram_width(K, prec)); }
+int part_rhs_of(int K, int prec) { return ntri(K > kNarrowMaxK ? K : gram_width(K, prec)); }
 int part_ld_of(int K, int prec) { return K > kNarrowMaxK ? wide_part_ld(K) : gram_part_ld(K, prec); }
 int part_parts(int K, int prec) { return K > kNarrowMaxK ? 1 : gram_parts(K, prec); }
 
@@ -482,7 +482,7 @@ bmf_status setup_side(bmf_ctx *c, Side &s, int64_t R, const std::vector<int64_t>
     const size_t nctr = s.h_multi.size() * (size_t)part_parts(c->K, c->prec);
     s.counters = c->mem.alloc<int>(nctr);
     s.multi_idx = c->mem.alloc<int32_t>(R);
-    s.rowsum = c->mem.alloc<double>(s.h_multi.size() * (size_t)part_nv(c->K));
+    s.rowsum = c->mem.alloc<double>(s.h_multi.size() * (size_t)part_nv(c->K, c->prec));
     if (!c->mem.ok) return fail(c, BMF_E_OOM, "device allocation failed (row sums)");
     CUDA_TRY(c, cudaMemset(s.counters, 0, std::max<size_t>(nctr, 1) * sizeof(int)));
     CUDA_TRY(c, cudaMemcpy(s.multi_idx, midx.data(), R * sizeof(int32_t), cudaMemcpyHostToDevice));
@@ -961,8 +961,8 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             gp.counters = me.counters;
             gp.nparts = part_parts(K, c->prec);
             gp.rowsum = me.rowsum;
-            gp.ld_sum = part_nv(K);
-            gp.nv = part_nv(K);
+            gp.ld_sum = part_nv(K, c->prec);
+            gp.nv = part_nv(K, c->prec);
             const int64_t b0 = me.slot_blk[sl0], b1 = me.slot_blk[sl1];
             // Gram pass over the rows of conditional blocks [ba, bb)
             auto gram_chunk = [&](int64_t ba, int64_t bb) {
@@ -982,7 +982,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
                     g.n_tasks = me.blk_task[bb] - me.blk_task[ba];
                     if (g.n_tasks > 0)
                         traced(c, c->st, f == 0 ? K_GRAM_X : K_GRAM_W, 1,
-                               [&] { launch_gram(K, c->prec, g, gram_grid, c->st); });
+                               [&] { launch_gram(c->prec, g, gram_grid, c->st); });
                 }
             };
             const std::vector<int64_t> &B = bounds[f];
@@ -1027,10 +1027,10 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             cp.item0 = i0;
             cp.part = c->part;
             cp.ld = c->ld_part;
-            cp.part_rhs = part_rhs_of(K);
+            cp.part_rhs = part_rhs_of(K, c->prec);
             cp.multi_idx = me.multi_idx;
             cp.rowsum = me.rowsum;
-            cp.ld_sum = part_nv(K);
+            cp.ld_sum = part_nv(K, c->prec);
             // sampled noise: the row side has the precisions in its Gram sums (scaled copies),
             // the column side takes each column's own
             cp.tau = c->noise ? 1.0 : c->tau;

@@ -7,10 +7,11 @@
 // one row per group).  Lanes of a group stride over the row's observations and gather one
 // partner row each with vector loads (the number of scattered load requests, not bytes, bounds
 // a gather on this GPU), accumulating the packed-lower Gram entries and the right-hand side in
-// registers; a butterfly reduce-scatter within the group then leaves each lane with a contiguous
-// slice of the summed entries, written with coalesced stores.  Entries are split into parts of
-// EP values when they do not fit in registers.  Rows longer than one item are finished by the
-// warp that completes their last item.  Every sum has a fixed order: results are deterministic.
+// registers; a butterfly
+// reduce-scatter within the group then leaves each lane with a slice of the summed entries.
+// Entries are split into parts of EP values when they do not fit in registers.  Rows longer than
+// one item are finished by the warp that completes their last item.  Every sum has a fixed order:
+// results are deterministic.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -29,21 +30,28 @@ int gather_ld(int K, int prec)
     return (KT + per16 - 1) / per16 * per16;
 }
 
-// Entries per part: registers hold EP accumulators per lane (FP32: up to 160, FP64: 32).
+// The latent dimension a kernel is compiled for: K itself in FP64, where the pass is bound by its
+// FP64 instructions (K = 5: 20 sums, 27 padded to K = 6: 54,000 rows of 74 observations 358 -> 265
+// us with the uneven reduce-scatter), K rounded up to an even number else.
+__host__ __device__ constexpr int width_of(int K, bool fp64) { return fp64 ? K : (K <= 1 ? 2 : (K + 1) / 2 * 2); }
+
+// Entries per part: FP32 registers hold all of a lane's accumulators (up to 160, in one part); FP64
+// takes as few equal parts of at most 32 as hold them (K = 10: 22 each; 32 + 32 + 1 gathered every
+// row a third time for one sum).
+__host__ __device__ constexpr int parts_of(int KT, bool fp64) { return fp64 ? (gram_nv(KT) + 31) / 32 : 1; }
 __host__ __device__ constexpr int ep_of(int KT, bool fp64)
 {
-    return fp64 ? 32 : (gram_nv(KT) <= 96 ? 96 : 160);
+    return fp64 ? (gram_nv(KT) + parts_of(KT, true) - 1) / parts_of(KT, true) : (gram_nv(KT) <= 96 ? 96 : 160);
 }
 
-static int ep_for(int KT, int prec) { return ep_of(KT, prec == BMF_FP64); }
+int gram_width(int K, int prec) { return width_of(K, prec == BMF_FP64); }
 
-int gram_parts(int K, int prec)
+int gram_parts(int K, int prec) { return parts_of(gram_width(K, prec), prec == BMF_FP64); }
+
+int gram_part_ld(int K, int prec)
 {
-    int KT = padded_k(K), ep = ep_for(KT, prec);
-    return (gram_nv(KT) + ep - 1) / ep;
+    return prec == BMF_FP64 ? (gram_nv(K) + 1) / 2 * 2 : ep_of(gram_width(K, prec), false);
 }
-
-int gram_part_ld(int K, int prec) { return gram_parts(K, prec) * ep_for(padded_k(K), prec); }
 
 // Lanes per row by its observation count: fewer lanes per row means more rows per warp and a
 // shorter reduce-scatter per row; measured on this GPU (69,878 x 10,677 Zipf workload, K = 10)
@@ -81,33 +89,30 @@ __device__ __forceinline__ void load_bits(const void *__restrict__ p, uint32_t (
     }
 }
 
-template <int KT>
-__device__ __forceinline__ void load_row(const float *__restrict__ p, float (&w)[KT])
+template <int K>
+__device__ __forceinline__ void load_row(const float *__restrict__ p, float (&w)[K])
 {
-    uint32_t u[KT];
-    load_bits<4 * KT>(p, u);
+    uint32_t u[K];
+    load_bits<4 * K>(p, u);
 #pragma unroll
-    for (int k = 0; k < KT; ++k) w[k] = __uint_as_float(u[k]);
+    for (int k = 0; k < K; ++k) w[k] = __uint_as_float(u[k]);
 }
-template <int KT>
-__device__ __forceinline__ void load_row(const double *__restrict__ p, double (&w)[KT])
+template <int K>
+__device__ __forceinline__ void load_row(const double *__restrict__ p, double (&w)[K])
 {
-    uint32_t u[2 * KT];
-    load_bits<8 * KT>(p, u);
+    uint32_t u[2 * K];
+    load_bits<8 * K>(p, u);
 #pragma unroll
-    for (int k = 0; k < KT; ++k) w[k] = __hiloint2double((int)u[2 * k + 1], (int)u[2 * k]);
+    for (int k = 0; k < K; ++k) w[k] = __hiloint2double((int)u[2 * k + 1], (int)u[2 * k]);
 }
-template <int KT>
-__device__ __forceinline__ void load_row(const __nv_bfloat16 *__restrict__ p, float (&w)[KT])
+template <int K>
+__device__ __forceinline__ void load_row(const __nv_bfloat16 *__restrict__ p, float (&w)[K])
 {
-    uint32_t u[KT / 2];
-    load_bits<2 * KT>(p, u);
+    uint32_t u[(K + 1) / 2];
+    load_bits<2 * K>(p, u);
 #pragma unroll
-    for (int k = 0; k < KT / 2; ++k) {
-        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u[k]));
-        w[2 * k] = f.x;
-        w[2 * k + 1] = f.y;
-    }
+    for (int k = 0; k < K; ++k)
+        w[k] = __uint_as_float(k & 1 ? u[k / 2] & 0xffff0000u : u[k / 2] << 16);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -137,6 +142,39 @@ __device__ __forceinline__ void rs_group(AT (&acc)[N], int lane)
     if constexpr (O >= 1) {
         rs_step<C, N, AT>(acc, lane, O);
         rs_group<C / 2, O / 2, N, AT>(acc, lane);
+    }
+}
+
+// The same for a count that need not divide (FP64, where every addition counts): the lanes with
+// bit O keep the upper values [H, C), the others the lower [0, H), H = ceil(C / 2); each adds its
+// partner's copy.  Afterwards a lane holds scattered<C, O>() values of the group's sums from
+// `base` on, those below `end`.
+template <int C, int O>
+__host__ __device__ constexpr int scattered()
+{
+    if constexpr (O >= 1)
+        return scattered<(C + 1) / 2, O / 2>();
+    else
+        return C;
+}
+template <int C, int O, int N, typename AT>
+__device__ __forceinline__ void rs_uneven(AT (&acc)[N], int lane, int &base, int &end)
+{
+    if constexpr (O >= 1) {
+        constexpr int H = (C + 1) / 2;
+        const bool up = (lane & O) != 0;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const AT lo = acc[i], hi = i + H < C ? acc[i + H < C ? i + H : 0] : AT(0);
+            const AT send = up ? lo : hi;
+            const AT keep = up ? hi : lo;
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+        }
+        if (up)
+            base += H;
+        else
+            end = min(end, base + H);
+        rs_uneven<H, O / 2, N, AT>(acc, lane, base, end);
     }
 }
 
@@ -179,11 +217,11 @@ __device__ __forceinline__ void gram_task(const GramParams &a, const GramTask &t
     const int64_t item = tk.item0 + (has ? g : 0);
     const GramItem m = a.items[item - a.item0];
     const int cnt = has ? m.count : 0;
-    // accumulators of this group width: the entries rounded up to a multiple of G (the
-    // reduce-scatter halves the set log2(G) times), not to the part width, when one part holds
-    // all of them
+    // accumulators of this group width: in FP32 the entries rounded up to a multiple of G (the
+    // reduce-scatter halves the set log2(G) times)
+    constexpr bool FP64 = sizeof(AT) == 8;
     constexpr int NV = gram_nv(KT);
-    constexpr int EPG = NV <= EP ? (NV + G - 1) / G * G : EP;
+    constexpr int EPG = FP64 ? EP : (NV + G - 1) / G * G;
     AT acc[EPG];
 #pragma unroll
     for (int v = 0; v < EPG; ++v) acc[v] = AT(0);
@@ -208,12 +246,21 @@ __device__ __forceinline__ void gram_task(const GramParams &a, const GramTask &t
         load_row<KT>(P + (int64_t)c * a.ldP, w);
         accum_all<KT, EPG, PART * EP, 0, AT>(acc, w, y);
     }
-    rs_group<EPG, G / 2, EPG, AT>(acc, lane);
-    constexpr int PER = EPG / G;
-    if (has) {
-        AT *dst = part + (item - a.item0) * (int64_t)a.ld + PART * EP + li * PER;
+    AT *dst = part + (item - a.item0) * (int64_t)a.ld + PART * EP;
+    if constexpr (FP64) {
+        int base = 0, end = NV - PART * EP < EP ? NV - PART * EP : EP;
+        rs_uneven<EPG, G / 2, EPG, AT>(acc, lane, base, end);
+        constexpr int PER = scattered<EPG, G / 2>();
 #pragma unroll
-        for (int v = 0; v < PER; ++v) dst[v] = acc[v];
+        for (int v = 0; v < PER; ++v)
+            if (has && base + v < end) dst[base + v] = acc[v];
+    } else {
+        rs_group<EPG, G / 2, EPG, AT>(acc, lane);
+        constexpr int PER = EPG / G;
+        if (has) {
+#pragma unroll
+            for (int v = 0; v < PER; ++v) dst[li * PER + v] = acc[v];
+        }
     }
     if constexpr (G == 32) {
         // A row split over several items: the warp that completes the row's last item sums all
@@ -247,10 +294,13 @@ __device__ __forceinline__ void gram_task(const GramParams &a, const GramTask &t
 template <int KT, typename GT, typename AT, int EP, int PART>
 __device__ __forceinline__ void gram_body(const GramParams &a)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // warp by warp within a block; fewer tasks than warps go to different blocks instead, so that
+    // they spread over the SMs
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t t = warp; t < a.n_tasks; t += nwarps) {
+    const bool few = a.n_tasks < nwarps;
+    for (int64_t t = few ? (int64_t)wib * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
+         t < a.n_tasks; t += nwarps) {
         const GramTask tk = a.tasks[t];
         if (tk.G == 8)
             gram_task<KT, GT, AT, EP, PART, 8>(a, tk, lane);
@@ -272,47 +322,41 @@ __device__ __forceinline__ void gram_dispatch(int part, const GramParams &a)
     }
 }
 
+constexpr int kGramThreads = 256;
+
 template <int KT, typename GT, typename AT, int EP>
-__global__ void __launch_bounds__(256, (EP > 96 ? 1 : 2)) gram_kernel(GramParams a)
+__global__ void __launch_bounds__(kGramThreads, (EP > 96 ? 1 : 2)) gram_kernel(GramParams a)
 {
-    constexpr int NP = (gram_nv(KT) + EP - 1) / EP;
-    gram_dispatch<KT, GT, AT, EP, 0, NP>(blockIdx.y, a);
+    gram_dispatch<KT, GT, AT, EP, 0, parts_of(KT, sizeof(AT) == 8)>(blockIdx.y, a);
 }
 
 template <int KT, typename GT, typename AT>
-static void launch_gram_t(const GramParams &a, int grid, int nparts, cudaStream_t st)
+static void launch_gram_t(const GramParams &a, int grid, cudaStream_t st)
 {
     constexpr int EP = ep_of(KT, sizeof(AT) == 8);
-    dim3 g(grid, nparts);
-    gram_kernel<KT, GT, AT, EP><<<g, 256, 0, st>>>(a);
+    const dim3 g(grid, parts_of(KT, sizeof(AT) == 8));
+    gram_kernel<KT, GT, AT, EP><<<g, kGramThreads, 0, st>>>(a);
 }
 
-template <typename GT, typename AT>
-static void launch_gram_k(int KT, const GramParams &a, int grid, int nparts, cudaStream_t st)
+template <int K, typename GT, typename AT>
+static void launch_gram_k(const GramParams &a, int grid, cudaStream_t st)
 {
-    switch (KT) {
-    case 2: launch_gram_t<2, GT, AT>(a, grid, nparts, st); break;
-    case 4: launch_gram_t<4, GT, AT>(a, grid, nparts, st); break;
-    case 6: launch_gram_t<6, GT, AT>(a, grid, nparts, st); break;
-    case 8: launch_gram_t<8, GT, AT>(a, grid, nparts, st); break;
-    case 10: launch_gram_t<10, GT, AT>(a, grid, nparts, st); break;
-    case 12: launch_gram_t<12, GT, AT>(a, grid, nparts, st); break;
-    case 14: launch_gram_t<14, GT, AT>(a, grid, nparts, st); break;
-    case 16: launch_gram_t<16, GT, AT>(a, grid, nparts, st); break;
-    default: break;
-    }
+    constexpr int KT = width_of(K, sizeof(AT) == 8);
+    if (width_of(a.K, sizeof(AT) == 8) == KT)
+        launch_gram_t<KT, GT, AT>(a, grid, st);
+    else if constexpr (K > 1)
+        launch_gram_k<K - 1, GT, AT>(a, grid, st);
 }
 
-void launch_gram(int K, int prec, const GramParams &a, int grid, cudaStream_t st)
+void launch_gram(int prec, const GramParams &a, int grid, cudaStream_t st)
 {
     if (a.n_tasks == 0) return;
-    const int KT = padded_k(K), np = gram_parts(K, prec);
     if (prec == BMF_FP64)
-        launch_gram_k<double, double>(KT, a, grid, np, st);
+        launch_gram_k<16, double, double>(a, grid, st);
     else if (prec == BMF_FP32)
-        launch_gram_k<float, float>(KT, a, grid, np, st);
+        launch_gram_k<16, float, float>(a, grid, st);
     else
-        launch_gram_k<__nv_bfloat16, float>(KT, a, grid, np, st);
+        launch_gram_k<16, __nv_bfloat16, float>(a, grid, st);
 }
 
 }  // namespace bmf

@@ -43,7 +43,9 @@ struct GramParams {
     int ld_sum;
     int nv;                    // entries per partial
 };
-void launch_gram(int K, int prec, const GramParams &a, int grid, cudaStream_t st);
+void launch_gram(int prec, const GramParams &a, int grid, cudaStream_t st);   // a.K <= 16
+// The latent dimension the K <= 16 Gram kernels are compiled for (their partials' layout).
+int gram_width(int K, int prec);
 int gram_parts(int K, int prec);
 
 // A block of the conditional kernel: up to 64 consecutive arena rows of one subset.
