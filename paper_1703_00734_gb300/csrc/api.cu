@@ -874,15 +874,18 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
     // (mu, Lambda) | factor for sweep `it`, on the side stream.  The statistics of X for sweep
     // it+1 depend only on the X written by sweep it, so they run while the main stream does
     // W | X of sweep it and the Gram pass of sweep it+1 (and symmetrically for W).
+    bool reduce[2] = {false, false};   // some job of the factor needs the first level of its sums
+    for (size_t q = 0; q < jobs.size(); ++q)
+        if (!direct_stats(K, jobs[q])) reduce[q < (size_t)nj[0] ? 0 : 1] = true;
     auto side_hyper = [&](int f, int it) -> bmf_status {
         const double *d = draws_of(it);
         if (bmf_status sw = wait_hyper(c->st2, it)) return sw;
         if (gen && it >= 2) CUDA_TRY(c, cudaStreamWaitEvent(c->st2, c->ev_gen[it & 1], 0));
         const int j0 = f == 0 ? 0 : nj[0];
-        HyperParams hp{K, c->d_jobs2 + j0, nj[f], c->stats2, c->mu0_d, c->beta0, c->nu0,
-                       c->W0inv_d, d, c->hyper, c->err_d};
-        traced(c, c->st2, K_HYPER, 2, [&] {
-            launch_stats_reduce(K, c->d_jobs + j0, nj[f], j0, c->stats, c->stats2, c->st2);
+        HyperParams hp{K, c->d_jobs + j0, nj[f], c->stats, c->d_jobs2 + j0, c->stats2, c->mu0_d, c->beta0,
+                       c->nu0, c->W0inv_d, d, c->hyper, c->err_d};
+        traced(c, c->st2, K_HYPER, reduce[f] ? 2 : 1, [&] {
+            if (reduce[f]) launch_stats_reduce(K, c->d_jobs + j0, nj[f], j0, c->stats, c->stats2, c->st2);
             launch_hyper(hp, c->st2);
         });
         CUDA_TRY(c, cudaEventRecord(c->ev_hyp[f], c->st2));

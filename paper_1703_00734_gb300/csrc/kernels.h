@@ -86,7 +86,7 @@ struct CondParams {
     double *stats;               // per-block sums of x and x x^T of the new state
                                  // [blocks x (K + ntri(K))], at slot blk0 + blockIdx.x
     int *parts_done;             // [blocks], zero between launches: a conditional block's rows may be
-                                 // split over several CUDA blocks (cond_parts), the last of which
+                                 // split over several CUDA blocks (grid y), the last of which
                                  // forms the block's statistics
     DevError *err;
     // rows marked kFusedRow in multi_idx form their own Gram sums from their observations (in
@@ -159,6 +159,8 @@ struct HyperParams {
     const HyperJob *jobs;
     int n_jobs;
     const double *stats;     // [chunks x (K + ntri)]
+    const HyperJob *jobs2;   // the same jobs over the first-level partials
+    const double *stats2;    // first-level partials (launch_stats_reduce)
     const double *mu0;       // [K]
     double beta0, nu0;
     const double *W0inv;     // [K*K]
@@ -169,6 +171,13 @@ struct HyperParams {
 void launch_hyper(const HyperParams &a, cudaStream_t st);
 // First level of the statistics sum: partials (j0 + j) * kStatParts + p of job j (see misc.cu).
 constexpr int kStatParts = 64;
+// A job of at most kStatParts chunks is summed by the draw itself, without the first level.  The rule
+// looks at the job alone, so its sums do not depend on the batch it is drawn in.  K > kPairsMaxK keeps
+// the first level for every job (its rounding: see hyper_kernel).
+__host__ __device__ inline bool direct_stats(int K, const HyperJob &j)
+{
+    return K <= kPairsMaxK && j.chunk1 - j.chunk0 <= kStatParts;
+}
 void launch_stats_reduce(int K, const HyperJob *jobs, int n_jobs, int j0, const double *stats,
                          double *out, cudaStream_t st);
 

@@ -93,9 +93,20 @@ void launch_stats(int K, const StatChunk *chunks, int n_chunks, const double *X,
 // Block-level dense FP64 linear algebra on K x K row-major matrices in shared memory.
 // ------------------------------------------------------------------------------------------
 
+// 1 / sqrt(d) to the last bit or two: the FP32 reciprocal square root and two Newton steps in FP64
+// (rsqrt_refined is the first), seven dependent FP64 operations; 0 < d, the CUDA function outside
+// the normal range.
+__device__ __forceinline__ double rsqrt_newton(double d)
+{
+    if (!pivot_ok(d)) return rsqrt(d);
+    const double y = rsqrt_refined(d);
+    return fma(0.5 * y, fma(-(d * y), y, 1.0), y);
+}
+
 // In-place lower Cholesky (right-looking); rinv[k] = 1 / L_kk.  Returns false (uniformly) if a
 // pivot is not > 0.  Two barriers per column: the trailing update of column k uses the unscaled
 // column times 1 / d_k, and column k is scaled during the next pivot step.
+template <bool FAST>
 __device__ bool block_chol(double *A, int K, double *rinv, int *flag)
 {
     const int t = threadIdx.x, T = blockDim.x;
@@ -105,7 +116,7 @@ __device__ bool block_chol(double *A, int K, double *rinv, int *flag)
             if (!(d > 0.0)) {
                 *flag = 1;
             } else {
-                const double r = rsqrt(d);
+                const double r = FAST ? rsqrt_newton(d) : rsqrt(d);
                 A[k * K + k] = d * r;
                 rinv[k] = r;
             }
@@ -134,7 +145,7 @@ __device__ bool block_chol(double *A, int K, double *rinv, int *flag)
 // First level of the statistics sum of the hyperparameter step: block (p, j) sums, entry by
 // entry in chunk order, the p-th of kStatParts equal runs of job j's chunks into partial
 // (j0 + j) * kStatParts + p (zero for an empty run).  The hyperparameter kernel then sums the
-// kStatParts partials of its job in order.
+// kStatParts partials of its job in order; jobs it sums from the chunks themselves are left out.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) stats_reduce_kernel(int K, const HyperJob *__restrict__ jobs,
                                                            int j0, const double *__restrict__ stats,
@@ -142,6 +153,7 @@ __global__ void __launch_bounds__(256) stats_reduce_kernel(int K, const HyperJob
 {
     const int NS = K + ntri(K);
     const HyperJob jb = jobs[blockIdx.y];
+    if (direct_stats(K, jb)) return;
     const int n = jb.chunk1 - jb.chunk0;
     const int len = (n + kStatParts - 1) / kStatParts;
     const int c0 = jb.chunk0 + min(n, (int)blockIdx.x * len), c1 = jb.chunk0 + min(n, ((int)blockIdx.x + 1) * len);
@@ -167,11 +179,22 @@ void launch_stats_reduce(int K, const HyperJob *jobs, int n_jobs, int j0, const 
 
 // ------------------------------------------------------------------------------------------
 // Normal-Wishart hyperparameter draw: one block per (subset, factor) job.
+//
+// The kernel is a chain of dependent FP64 operations (64 clocks each) on the path from one sweep to
+// the next: FAST shortens it where small problems wait for it (the pivots' reciprocal square roots
+// by Newton steps, reciprocals computed while the statistics load, the triangular solve by a warp).
+// K > kPairsMaxK keeps the plain operations: its draws hide the chain, and there a change of
+// rounding moves a reduced-precision chain too far (cond_pairs.cu).  K = 10, 1,000 rows, with the
+// statistics sum: 41 us, 29 us FAST.
 // ------------------------------------------------------------------------------------------
+template <bool FAST>
 __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
 {
-    const HyperJob jb = a.jobs[blockIdx.x];
-    const int K = a.K, KK = K * K, NS = K + ntri(K);
+    const int K = a.K;
+    const bool direct = direct_stats(K, a.jobs[blockIdx.x]);
+    const HyperJob jb = (direct ? a.jobs : a.jobs2)[blockIdx.x];
+    const double *stats = direct ? a.stats : a.stats2;
+    const int KK = K * K, NS = K + ntri(K);
     const int t = threadIdx.x, T = blockDim.x;
     extern __shared__ double s[];
     double *M = s, *C = M + KK, *L = C + KK, *B = L + KK;
@@ -180,6 +203,9 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
     double *red = rinv + K;  // [T] stripe partial sums
     __shared__ int flag;
     if (t == 0) flag = 0;
+    const double N = (double)jb.n;
+    const double bstar = a.beta0 + N;
+    const double inv_n = FAST && N > 0 ? 1.0 / N : 0.0, inv_b = FAST ? 1.0 / bstar : 0.0;
     // 1. sum the chunk statistics: each entry is split over `ns` stripes of chunks, each
     //    stripe summed with eight independent accumulators, then the stripes in order (a fixed
     //    order for a given block size, so the result is deterministic)
@@ -190,9 +216,9 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
         int c = jb.chunk0 + sidx;
         for (; c + 7 * ns < jb.chunk1; c += 8 * ns) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] += a.stats[(int64_t)(c + u * ns) * NS + e];
+            for (int u = 0; u < 8; ++u) acc[u] += stats[(int64_t)(c + u * ns) * NS + e];
         }
-        for (; c < jb.chunk1; c += ns) acc[0] += a.stats[(int64_t)c * NS + e];
+        for (; c < jb.chunk1; c += ns) acc[0] += stats[(int64_t)c * NS + e];
         const double part = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
         if (ns > 1)
             red[q] = part;
@@ -221,20 +247,27 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
         }
         __syncthreads();
     }
-    const double N = (double)jb.n;
-    const double bstar = a.beta0 + N;
     for (int e = t; e < K; e += T) {
-        xbar[e] = N > 0 ? s1[e] / N : 0.0;
-        mus[e] = (a.beta0 * a.mu0[e] + N * (N > 0 ? s1[e] / N : 0.0)) / bstar;
+        if constexpr (FAST) {
+            xbar[e] = s1[e] * inv_n;
+            mus[e] = fma(a.beta0, a.mu0[e], s1[e]) * inv_b;
+        } else {
+            xbar[e] = N > 0 ? s1[e] / N : 0.0;
+            mus[e] = (a.beta0 * a.mu0[e] + N * (N > 0 ? s1[e] / N : 0.0)) / bstar;
+        }
     }
     __syncthreads();
     // 2. [W*]^{-1} = W0^{-1} + N Sbar + (beta0 N / beta*) (mu0 - xbar)(mu0 - xbar)^T with the
     //    centred Sbar = (1/N) sum x x^T - xbar xbar^T
-    const double cw = a.beta0 * N / bstar;
+    const double cw = FAST ? a.beta0 * N * inv_b : a.beta0 * N / bstar;
     for (int e = t; e < KK; e += T) {
         const int i = e / K, j = e % K;
-        const double Sb = N > 0 ? M[e] / N - xbar[i] * xbar[j] : 0.0;
-        C[e] = a.W0inv[e] + N * Sb + cw * (a.mu0[i] - xbar[i]) * (a.mu0[j] - xbar[j]);
+        double NSb;   // N Sbar
+        if constexpr (FAST)
+            NSb = fma(-s1[i], xbar[j], M[e]);
+        else
+            NSb = N * (N > 0 ? M[e] / N - xbar[i] * xbar[j] : 0.0);
+        C[e] = a.W0inv[e] + NSb + cw * (a.mu0[i] - xbar[i]) * (a.mu0[j] - xbar[j]);
     }
     __syncthreads();
     // 3. the lower Cholesky factor of W* = ([W*]^{-1})^{-1} without forming W*: with P the
@@ -242,16 +275,21 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
     //    and P R^{-T} P is lower with a positive diagonal, so it is that factor
     for (int e = t; e < KK; e += T) L[e] = C[(KK - 1) - e];
     __syncthreads();
-    if (!block_chol(L, K, rinv, &flag)) goto fail;
-    for (int c = t; c < K; c += T) {           // R^{-1} (lower) into M, a column per thread
-        for (int i = 0; i < c; ++i) M[i * K + c] = 0.0;
-        for (int i = c; i < K; ++i) {
-            double acc = i == c ? 1.0 : 0.0;
-            for (int k = c; k < i; ++k) acc = fma(-L[i * K + k], M[k * K + c], acc);
-            M[i * K + c] = acc * rinv[i];
-        }
-    }
+    if (!block_chol<FAST>(L, K, rinv, &flag)) goto fail;
+    // R^{-1} (lower) into M: row i scaled, then taken from the rows below (per entry the operations of
+    // a column's forward substitution in its order), a row of the rest per warp pass
+    for (int e = t; e < KK; e += T) M[e] = e / K == e % K ? 1.0 : 0.0;
     __syncthreads();
+    for (int i = 0; i < K; ++i) {
+        for (int c = t; c <= i; c += T) M[i * K + c] *= rinv[i];
+        __syncthreads();
+        const int w = i + 1;
+        for (int e = t; e < (K - 1 - i) * w; e += T) {
+            const int r = i + 1 + e / w, c = e % w;
+            M[r * K + c] = fma(-L[r * K + i], M[i * K + c], M[r * K + c]);
+        }
+        __syncthreads();
+    }
     // 4. L = P R^{-T} P: L_ij = (R^{-1})_{K-1-j, K-1-i}
     for (int e = t; e < KK; e += T) {
         const int i = e / K, j = e % K;
@@ -300,7 +338,20 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
     }
     __syncthreads();
     if (flag) goto fail;
-    if (t == 0) {
+    if constexpr (FAST) {
+        if (t < 32) {   // column by column, lane l holding v_l and v_{l + 32}
+            double v0 = t < K ? v[t] : 0.0, v1 = t + 32 < K ? v[t + 32] : 0.0;
+            for (int i = K - 1; i >= 0; --i) {
+                const double x = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31) * rinv[i];
+                if (t == (i & 31)) (i < 32 ? v0 : v1) = x;
+                if (t < i) v0 = fma(-C[i * K + t], x, v0);
+                if (t + 32 < i) v1 = fma(-C[i * K + t + 32], x, v1);
+            }
+            const double sb = rsqrt_newton(bstar);
+            if (t < K) mu[t] = fma(v0, sb, mus[t]);
+            if (t + 32 < K) mu[t + 32] = fma(v1, sb, mus[t + 32]);
+        }
+    } else if (t == 0) {
         const double sb = rsqrt(bstar);
         for (int i = K - 1; i >= 0; --i) {
             double acc = v[i];
@@ -330,13 +381,22 @@ fail:
     if (t == 0) atomicOr(&a.err->flags, ERR_NOT_PD);
 }
 
+template <bool FAST>
+static void launch_hyper_t(const HyperParams &a, cudaStream_t st)
+{
+    const size_t smem = (size_t)(4 * a.K * a.K + 6 * a.K + 256) * sizeof(double);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(hyper_kernel<FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    hyper_kernel<FAST><<<a.n_jobs, 256, smem, st>>>(a);
+}
+
 void launch_hyper(const HyperParams &a, cudaStream_t st)
 {
     if (a.n_jobs <= 0) return;
-    const size_t smem = (size_t)(4 * a.K * a.K + 6 * a.K + 256) * sizeof(double);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(hyper_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    hyper_kernel<<<a.n_jobs, 256, smem, st>>>(a);
+    if (a.K <= kPairsMaxK)
+        launch_hyper_t<true>(a, st);
+    else
+        launch_hyper_t<false>(a, st);
 }
 
 // ------------------------------------------------------------------------------------------
