@@ -466,14 +466,19 @@ void launch_gram_wide(int K, int prec, const GramParams &a, int grid, cudaStream
 // 32 above), 32 / T rows per warp at a time; below K = 13 one thread per row (cond.cu) is as
 // fast.  Measured on this GPU: equal at K = 10, the team form 18% faster at K = 16; at K = 32
 // teams of 16 lanes 7% faster than teams of 8 and 20% faster than 32.
-// The row's packed matrix lives in shared memory; the team factors it right-looking (each step:
-// the pivot, read by every lane, then the column scaled and the trailing triangle updated with
-// the entries spread over the team), then solves column by column.  On this GPU the FP64 pipe
-// issues one warp instruction every few dozen cycles per SM partition, so the pivot chain
-// (square root, reciprocal) is what one row costs serially; several rows per warp share it,
-// while the O(K^3) trailing updates keep all lanes busy.  Every team of a warp runs the same
-// number of steps (rows beyond the block and rows that fail the positive-definiteness test
-// still run the loop structure), and synchronisation is per team.
+// The row's matrix lives in shared memory; the team factors it right-looking (each step: the
+// pivot, read by every lane, then the column scaled and the trailing triangle updated with the
+// entries spread over the team), with the right-hand side as one more row, so that the forward
+// solve is part of the same updates, then solves backwards column by column.  On this GPU the FP64
+// pipe issues one warp instruction every 16 cycles per SM, so what bounds a row is the FP64 warp
+// instructions it issues (1,900 at K = 64, 1,330 of them trailing updates), if each warp can issue
+// the rest between them: few warps fit beside their matrices (12 per SM at K = 64).  Walking the
+// rows of a row-packed triangle took 30 instructions per update and left the pipe at 69%; column by
+// column the trailing matrix is one run, and a table gives the row and column of its entries
+// (K = 64, 50,000 rows: 8.06 ms before, 6.89 ms now).  Several rows per warp share the pivot chain
+// where they fit.  Every team of a warp runs the same number of steps (rows beyond the block and
+// rows that fail the positive-definiteness test still run the loop structure), and synchronisation
+// is per team.
 // ------------------------------------------------------------------------------------------
 template <typename GT>
 __device__ __forceinline__ GT to_gather_w(double x);
@@ -506,26 +511,36 @@ __device__ __forceinline__ void decode_packed(int e, int &i, int &j)
 // 1.10 ms per stage-3 X half against 1.33 ms for four-lane teams.
 int cond_team_size(int K) { return K <= 16 ? 2 : (K <= 48 ? 16 : 32); }
 
-// Doubles per team in shared memory: the packed matrix, right-hand side, pivots and (teams of 8
-// or more lanes) a contiguous copy of the current column, rounded up to a multiple of 8 doubles
-// and offset by T mod 16 doubles (4 for teams of 16 or 32 lanes), so that consecutive teams of
-// a warp start in different banks.  Rounding to 8 rather than 16 doubles lets five blocks of
-// 4-lane teams share an SM at K = 16 (44 KB each).  The column copy removes the strided reads of
-// the trailing update; for 4-lane teams (K <= 16) the extra shared memory would cost a resident
-// block per SM, which measured slower.
-__host__ __device__ constexpr bool team_colcopy(int T) { return T >= 8; }
+// Doubles per team in shared memory: the lower triangle of [Lambda, b; b^T] without its last corner,
+// column by column (column j: rows j..K, row K being b), rounded up to a multiple of 8 doubles and
+// offset by T mod 16 doubles (4 for teams of 16 or 32 lanes), so that consecutive teams of a warp
+// start in different banks.  In this order the trailing matrix of a step is one contiguous run and
+// so is the column it is updated with.  1 / L_kk takes the place of the diagonal.
 __host__ __device__ constexpr int team_stride(int K, int T)
 {
-    return (ntri(K) + (team_colcopy(T) ? 3 : 2) * K + 7) / 8 * 8 + (T % 16 == 0 ? 4 : T % 16);
+    return (ntri(K) + K + 7) / 8 * 8 + (T % 16 == 0 ? 4 : T % 16);
+}
+__host__ __device__ constexpr int col_base(int K, int j) { return j * (K + 1) - j * (j - 1) / 2; }
+// A block's shared memory: its teams' matrices, then row and column of each packed entry (16 bits)
+__host__ __device__ constexpr size_t team_smem(int K, int T)
+{
+    return (size_t)(32 * kWideWarps / T) * team_stride(K, T) * sizeof(double) + (size_t)(ntri(K) + K) * sizeof(uint16_t);
 }
 
+// The lanes a schedule may ask for: teams whose matrices, right-hand sides, pivots and (8 lanes or
+// more) a column fit in a block's shared memory, a little more than team_smem.
 bool cond_lanes_valid(int K, int lanes)
 {
     if (lanes == 2 && K >= 13 && K <= 16) return true;
     if (lanes != 2 && lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32) return false;
-    const size_t smem = (size_t)(32 * kWideWarps / lanes) * team_stride(K, lanes) * sizeof(double);
-    return smem <= 227 * 1024;
+    const int doubles = (ntri(K) + (lanes >= 8 ? 3 : 2) * K + 7) / 8 * 8 + (lanes % 16 == 0 ? 4 : lanes % 16);
+    return (size_t)(32 * kWideWarps / lanes) * doubles * sizeof(double) <= 227 * 1024;
 }
+
+// Entries of a lane in flight in the assembly and the trailing updates: few warps fit beside their
+// matrices (three per scheduler at K = 64), so one warp alone has to keep its FP64 pipe busy while
+// the others wait for loads or a pivot.
+constexpr int kTeamBatch = 4;
 
 template <typename GT, typename AT, int T>
 __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a)
@@ -535,8 +550,13 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
     const int K = a.K, NT = ntri(K);
     const int tl = threadIdx.x % T, tm = threadIdx.x / T;
     const unsigned mask = T == 32 ? 0xffffffffu : (((1u << T) - 1u) << ((threadIdx.x & 31) & ~(T - 1)));
-    const int per_team = team_stride(K, T);
-    double *M = smw + tm * per_team, *B = M + NT, *RI = B + K, *CK = RI + K;
+    const int E = NT + K;   // entries of a matrix
+    double *M = smw + tm * team_stride(K, T);
+    auto at = [K](int i, int j) { return col_base(K, j) + i - j; };   // row i, column j <= i
+    uint16_t *tab = reinterpret_cast<uint16_t *>(smw + NTEAM * team_stride(K, T));
+    for (int j = threadIdx.x / 32; j < K; j += kWideWarps)
+        for (int i = j + (threadIdx.x & 31); i <= K; i += 32) tab[at(i, j)] = (uint16_t)(i << 8 | j);
+    __syncthreads();
     const CondBlock blk = a.blocks[blockIdx.x];
     const int64_t R = a.R;
     const double tau = a.tau;
@@ -554,12 +574,14 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
             const AT *pp = static_cast<const AT *>(a.part) + (i0 - a.item0) * (int64_t)a.ld;
             const double *ps = mi >= 0 ? a.rowsum + (int64_t)mi * a.ld_sum : nullptr;
             const double tau_r = a.tau_row ? a.tau_row[r] : tau;
-            for (int e = tl; e < NT + K; e += T) {
-                const int src = e < NT ? e : a.part_rhs + (e - NT);
-                double gsum;
-                if (mi == kFusedRow) {
-                    // a row with few observations: the entry from its list, in list order (the
-                    // same operations as the two-lane conditional)
+            auto prior = [&](int e) {   // e: packed entry, then NT + i
+                if (hp) return hp[K + e];
+                return e < NT ? a.prior_L[(int64_t)e * R + r] : a.prior_b[(int64_t)(e - NT) * R + r];
+            };
+            if (mi == kFusedRow) {
+                // a row with few observations: each entry from its list, in list order (the same
+                // operations as the two-lane conditional)
+                for (int e = tl; e < E; e += T) {
                     int ii, jj;
                     if (e < NT)
                         decode_packed(e, ii, jj);
@@ -572,55 +594,66 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
                         acc = jj >= 0 ? acc_fma(pi, to_acc<AT>(pr[jj]), acc)
                                       : acc_fma(static_cast<const AT *>(a.obs_val)[o], pi, acc);
                     }
-                    gsum = widen(acc);
-                } else {
-                    gsum = ps ? ps[src] : (i1 > i0 ? widen(pp[src]) : 0.0);
+                    M[jj >= 0 ? at(ii, jj) : at(K, ii)] = fma(tau_r, widen(acc), prior(e));
                 }
-                double prior;
-                if (e < NT)
-                    prior = hp ? hp[K + e] : a.prior_L[(int64_t)e * R + r];
-                else
-                    prior = hp ? hp[K + NT + (e - NT)] : a.prior_b[(int64_t)(e - NT) * R + r];
-                M[e] = fma(tau_r, gsum, prior);   // M[NT + i] is B[i]
+            } else {
+                const bool one = ps == nullptr && i1 > i0;
+                int i = 0, j = tl;   // row and column of the packed rows' entry e0 (row K: b)
+                for (int e0 = tl; e0 < E; e0 += kTeamBatch * T) {
+                    double g[kTeamBatch], p[kTeamBatch];
+#pragma unroll
+                    for (int u = 0; u < kTeamBatch; ++u) {
+                        const int e = min(e0 + u * T, E - 1);
+                        const int src = e < NT ? e : a.part_rhs + (e - NT);
+                        g[u] = ps ? ps[src] : (one ? widen(pp[src]) : 0.0);
+                        p[u] = prior(e);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kTeamBatch; ++u) {
+                        while (i < K && j > i) {
+                            ++i;
+                            j -= i;
+                        }
+                        if (e0 + u * T < E) M[at(i, j)] = fma(tau_r, g[u], p[u]);
+                        j += T;
+                    }
+                }
             }
         }
         __syncwarp(mask);
-        // 3. right-looking Cholesky
+        // 3-4. right-looking Cholesky of [Lambda, b; b^T]: the last row of the factor is y with
+        // L y = b, formed by the same updates
         bool ok = active;
         for (int k = 0; k < K; ++k) {
-            const int kk = tri(k, k);
-            const double d = ok ? M[kk] : 1.0;
+            double *col = M + col_base(K, k) - k;   // column k by row
+            const double d = ok ? col[k] : 1.0;
             if (!pivot_ok(d)) ok = false;
             const double rs = ok ? pivot_rsqrt<GT>(d) : 0.0;
             __syncwarp(mask);
             if (ok) {
-                // the scaled column also goes to CK[i], contiguous, for the trailing update
-                for (int i = k + 1 + tl; i < K; i += T) {
-                    const double l = M[tri(i, k)] * rs;
-                    M[tri(i, k)] = l;
-                    if constexpr (team_colcopy(T)) CK[i] = l;
-                }
-                if (tl == 0) RI[k] = rs;   // the solves scale by 1 / L_kk; L_kk itself is not kept
+                for (int i = k + 1 + tl; i <= K; i += T) col[i] *= rs;
+                if (tl == 0) col[k] = rs;   // the solve scales by 1 / L_kk; L_kk itself is not kept
             }
             __syncwarp(mask);
             if (ok) {
-                // trailing triangle rows i = k+1..K-1, columns j = k+1..i, row by row; lane tl
-                // takes positions tl, tl + T, ... (row i holds i - k of them)
-                int i = k + 1, j = k + 1 + tl;
-                while (i < K && j > i) {
-                    j -= i - k;
-                    ++i;
-                }
-                while (i < K) {
-                    if constexpr (team_colcopy(T))
-                        M[tri(i, j)] = fma(-CK[i], CK[j], M[tri(i, j)]);
-                    else
-                        M[tri(i, j)] = fma(-M[tri(i, k)], M[tri(j, k)], M[tri(i, j)]);
-                    j += T;
-                    while (i < K && j > i) {
-                        j -= i - k;
-                        ++i;
+                // the trailing matrix, entries s + tl, s + T + tl, ...: kTeamBatch at a time, then
+                // the rest
+                int s = col_base(K, k + 1);
+                for (; s + kTeamBatch * T <= E; s += kTeamBatch * T) {
+                    double m[kTeamBatch], p[kTeamBatch], q[kTeamBatch];
+#pragma unroll
+                    for (int u = 0; u < kTeamBatch; ++u) {
+                        const int ij = tab[s + tl + u * T];
+                        m[u] = M[s + tl + u * T];
+                        p[u] = col[ij >> 8];
+                        q[u] = col[ij & 255];
                     }
+#pragma unroll
+                    for (int u = 0; u < kTeamBatch; ++u) M[s + tl + u * T] = fma(-p[u], q[u], m[u]);
+                }
+                for (s += tl; s < E; s += T) {
+                    const int ij = tab[s];
+                    M[s] = fma(-col[ij >> 8], col[ij & 255], M[s]);
                 }
             }
             __syncwarp(mask);
@@ -629,28 +662,22 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
             atomicOr(&a.err->flags, ERR_NOT_PD);
             atomicMin(&a.err->first_bad_row, (int)r);
         }
-        // 4. forward solve L y = b (column oriented)
-        for (int k = 0; k < K; ++k) {
-            const double yk = ok ? B[k] * RI[k] : 0.0;
-            __syncwarp(mask);
-            if (ok) {
-                for (int i = k + 1 + tl; i < K; i += T) B[i] = fma(-M[tri(i, k)], yk, B[i]);
-                if (tl == 0) B[k] = yk;
-            }
-            __syncwarp(mask);
-        }
-        // 5. back solve L^T x = y + z (column oriented)
+        // 5. back solve L^T x = y + z (column oriented), x in the place of y
+        auto B = [&](int i) -> double & { return M[at(K, i)]; };
         if (ok) {
             const double *z = a.z + (r - a.row0) * K;
-            for (int i = tl; i < K; i += T) B[i] += z[i];
+            for (int i = tl; i < K; i += T) B(i) += z[i];
         }
         __syncwarp(mask);
         for (int i = K - 1; i >= 0; --i) {
-            const double xi = ok ? B[i] * RI[i] : 0.0;
+            const double xi = ok ? B(i) * M[at(i, i)] : 0.0;
             __syncwarp(mask);
             if (ok) {
-                for (int k = tl; k < i; k += T) B[k] = fma(-M[tri(i, k)], xi, B[k]);
-                if (tl == 0) B[i] = xi;
+                for (int k = tl; k < i; k += T) {
+                    double *col = M + col_base(K, k) - k;
+                    col[K] = fma(-col[i], xi, col[K]);
+                }
+                if (tl == 0) B(i) = xi;
             }
             __syncwarp(mask);
         }
@@ -658,7 +685,7 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
         if (active) {
             GT *g = static_cast<GT *>(a.Xg) + r * a.ldg;
             for (int i = tl; i < a.ldg; i += T) {
-                const double xi = (ok && i < K) ? B[i] : 0.0;
+                const double xi = (ok && i < K) ? B(i) : 0.0;
                 if (ok) g[i] = to_gather_w<GT>(xi);
                 if (i < K && ok) {
                     a.X[r * K + i] = xi;
@@ -669,7 +696,7 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
                 for (int e = tl; e < NT; e += T) {
                     int i, j;
                     decode_packed(e, i, j);
-                    a.S2[(int64_t)e * R + r] += B[i] * B[j];
+                    a.S2[(int64_t)e * R + r] += B(i) * B(j);
                 }
         }
         __syncwarp(mask);
@@ -701,10 +728,10 @@ template <typename GT, typename AT, int T>
 static void launch_cond_team_t(const CondParams &a, int n_blocks, int sms, cudaStream_t st)
 {
     constexpr int NTEAM = 32 * kWideWarps / T;
-    const size_t smem = (size_t)NTEAM * team_stride(a.K, T) * sizeof(double);
+    const size_t smem = team_smem(a.K, T);
     // parts of at least a round's rows, until the launch fills the GPU about eight times over
-    // (K = 64: 12,500 rows, 196 blocks, 4.27 ms as one part, 2.08 ms in parts; 50,000 rows 9.17 and
-    // 8.08 ms)
+    // (K = 64, before the column layout: 12,500 rows, 196 blocks, 4.27 ms as one part, 2.08 ms in
+    // parts, 1.78 ms now; 50,000 rows 9.17 and 8.08 ms)
     const int per_sm = (int)std::max<size_t>(1, (size_t)220 * 1024 / smem);
     int parts = 1;
     while (parts < kCondBlock / NTEAM && (int64_t)n_blocks * parts < (int64_t)8 * sms * per_sm) parts *= 2;
