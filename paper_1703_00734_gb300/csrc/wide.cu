@@ -489,15 +489,6 @@ __device__ __forceinline__ float to_gather_w<float>(double x) { return (float)x;
 template <>
 __device__ __forceinline__ __nv_bfloat16 to_gather_w<__nv_bfloat16>(double x) { return __double2bfloat16(x); }
 
-template <typename AT>
-__device__ __forceinline__ AT to_acc(double x) { return x; }
-template <typename AT>
-__device__ __forceinline__ AT to_acc(float x) { return x; }
-template <typename AT>
-__device__ __forceinline__ AT to_acc(__nv_bfloat16 x) { return __bfloat162float(x); }
-__device__ __forceinline__ float acc_fma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double acc_fma(double a, double b, double c) { return fma(a, b, c); }
-
 __device__ __forceinline__ void decode_packed(int e, int &i, int &j)
 {
     i = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
@@ -578,23 +569,22 @@ __global__ void __launch_bounds__(32 * kWideWarps) cond_team_kernel(CondParams a
                 if (hp) return hp[K + e];
                 return e < NT ? a.prior_L[(int64_t)e * R + r] : a.prior_b[(int64_t)(e - NT) * R + r];
             };
-            if (mi == kFusedRow) {
-                // a row with few observations: each entry from its list, in list order (the same
-                // operations as the two-lane conditional)
+            if (sizeof(GT) == 8 && mi == kFusedRow) {
+                // a row with few observations (K <= 16): each entry from its list, in list order
+                // (the same operations as the two-lane conditional)
+                const double *P = static_cast<const double *>(a.P), *val = static_cast<const double *>(a.obs_val);
                 for (int e = tl; e < E; e += T) {
                     int ii, jj;
                     if (e < NT)
                         decode_packed(e, ii, jj);
                     else
                         ii = e - NT, jj = -1;
-                    AT acc = AT(0);
+                    double acc = 0.0;
                     for (int64_t o = a.obs_ptr[r]; o < a.obs_ptr[r + 1]; ++o) {
-                        const GT *pr = static_cast<const GT *>(a.P) + (int64_t)a.obs_idx[o] * a.ldP;
-                        const AT pi = to_acc<AT>(pr[ii]);
-                        acc = jj >= 0 ? acc_fma(pi, to_acc<AT>(pr[jj]), acc)
-                                      : acc_fma(static_cast<const AT *>(a.obs_val)[o], pi, acc);
+                        const double *pr = P + (int64_t)a.obs_idx[o] * a.ldP;
+                        acc = jj >= 0 ? fma(pr[ii], pr[jj], acc) : fma(val[o], pr[ii], acc);
                     }
-                    M[jj >= 0 ? at(ii, jj) : at(K, ii)] = fma(tau_r, widen(acc), prior(e));
+                    M[jj >= 0 ? at(ii, jj) : at(K, ii)] = fma(tau_r, acc, prior(e));
                 }
             } else {
                 const bool one = ps == nullptr && i1 > i0;
@@ -743,9 +733,12 @@ static void launch_cond_team_t(const CondParams &a, int n_blocks, int sms, cudaS
 template <typename GT, typename AT>
 static void launch_cond_team_p(const CondParams &a, int n_blocks, int team, int sms, cudaStream_t st)
 {
+    // (2 or 4 lanes fit up to K = 40, where the reduced-precision modes draw in pairs)
+    if constexpr (sizeof(GT) == 8) {
+        if (team == 2) return launch_cond_team_t<GT, AT, 2>(a, n_blocks, sms, st);
+        if (team == 4) return launch_cond_team_t<GT, AT, 4>(a, n_blocks, sms, st);
+    }
     switch (team) {
-    case 2: launch_cond_team_t<GT, AT, 2>(a, n_blocks, sms, st); break;
-    case 4: launch_cond_team_t<GT, AT, 4>(a, n_blocks, sms, st); break;
     case 8: launch_cond_team_t<GT, AT, 8>(a, n_blocks, sms, st); break;
     case 16: launch_cond_team_t<GT, AT, 16>(a, n_blocks, sms, st); break;
     default: launch_cond_team_t<GT, AT, 32>(a, n_blocks, sms, st); break;
