@@ -41,7 +41,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 WORKLOAD = "pp4x4-100000x20000-20M-k16"
-# arithmetic of the path per --precision: gathers and Gram sums, then the FP64 conditional
+# arithmetic of the path per --precision: gathers and Gram sums, then the FP64 rest (at 9 <= K <= 48
+# the reduced-precision modes draw from the conditionals in float pairs of 48 bits)
 DTYPE = {"fp32": "f32+f64", "bf16": "bf16+f64", "tf32": "tf32+f64", "fp64": "f64"}
 PLAIN_WORKLOAD = "zipf-69878x10677-10M-k10"
 METRIC = "Gibbs sweeps/s"
@@ -49,6 +50,16 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # FP64 ALU peak: 152 SMs x 2 FP64 FMA/clock x 2 FLOP x 2.07 GHz (unit count and maximum clock
 # of this GPU; a dependent-free DFMA loop measured 1.19 TFLOP/s, 1.89 FMA/clock/SM).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+# The same multiply-adds in float pairs: twelve FP32 instructions each, four warp instructions per
+# clock and SM.
+PAIR_PEAK_TFLOPS = 152 * 128 / 12 * 2 * 2.07e9 / 1e12
+
+
+def alu_peak(K, prec):
+    """Peak of the conditional draws (TFLOP/s) and where it comes from."""
+    if prec != "fp64" and 9 <= K <= 48:
+        return PAIR_PEAK_TFLOPS, "derived: 152 SMs x 128 FP32 FMA/clk / 12 per pair FMA x 2 x 2.07 GHz"
+    return FP64_PEAK_TFLOPS, "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz"
 
 
 def log(*a):
@@ -301,7 +312,7 @@ def run_ours(args, rank, world, local_rank):
         if name in algo:
             bound, work, unit = algo[name]
             ach = work / (avg_ms / 1e3) / (1e9 if unit == "GB/s" else 1e12)
-            peak = hbm if unit == "GB/s" else FP64_PEAK_TFLOPS
+            peak = hbm if unit == "GB/s" else alu_peak(K, args.precision)[0]
             ent.update(bound=bound, achieved=ach, peak=peak, unit=unit, frac=ach / peak)
         kernels[name] = ent
     total = sum(v["avg_us"] * v["launches"] for v in kernels.values())
@@ -313,7 +324,7 @@ def run_ours(args, rank, world, local_rank):
     roof = {"kernel": dom, "bound": kd["bound"], "achieved": kd["achieved"], "peak": kd["peak"],
             "unit": kd["unit"], "frac": kd["frac"], "traffic": traffic_for(dom, args.precision, args.workload),
             "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if kd["unit"] == "GB/s"
-            else "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz"}
+            else alu_peak(K, args.precision)[1]}
     out = {
         "metric": METRIC, "value": sweeps_s, "unit": "sweeps/s", "n_gpus": world, "steps": S,
         "warmup": W, "ms_per_step": ms / S, "higher_is_better": True, "scaling": "weak",
@@ -382,7 +393,7 @@ def pp_algorithmic(geom, K, prec):
     return out
 
 
-def pp_kernel_table(prof_by_stage, algo, hbm):
+def pp_kernel_table(prof_by_stage, algo, hbm, alu=FP64_PEAK_TFLOPS):
     """Per (stage, kernel class): launches, mean launch time and, for the Gram and conditional
     classes, achieved work against the peak.  `stream_time_share` is the class's summed launch
     time over the summed time of all classes: classes on side streams (hyperparameter draws,
@@ -398,7 +409,7 @@ def pp_kernel_table(prof_by_stage, algo, hbm):
             if (st, name) in algo:
                 bound, work, unit = algo[(st, name)]
                 ach = work / (t / n / 1e3) / (1e9 if unit == "GB/s" else 1e12)
-                peak = hbm if unit == "GB/s" else FP64_PEAK_TFLOPS
+                peak = hbm if unit == "GB/s" else alu
                 ent.update(bound=bound, work_per_launch=work, achieved=ach, peak=peak,
                            unit=unit, frac=ach / peak)
             rows[f"s{st}.{name}"] = ent
@@ -582,7 +593,7 @@ def run_pp(args, rank, world, local_rank):
     peaks = json.load(open(PEAKS_FILE)) if os.path.exists(PEAKS_FILE) else {}
     hbm = peaks.get("hbm_gbs", 6800.0)
     algo = pp_algorithmic(geom, K, args.precision)
-    kernels = pp_kernel_table(prof_by_stage, algo, hbm)
+    kernels = pp_kernel_table(prof_by_stage, algo, hbm, alu_peak(K, args.precision)[0])
     dom = max((k for k in kernels if "bound" in kernels[k]),
               key=lambda k: kernels[k]["avg_us"] * kernels[k]["launches"])
     kd = kernels[dom]
@@ -591,7 +602,7 @@ def run_pp(args, rank, world, local_rank):
             "traffic": traffic_for(dom, args.precision, args.workload),
             "work_per_launch": kd["work_per_launch"],
             "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if kd["unit"] == "GB/s"
-            else "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz"}
+            else alu_peak(K, args.precision)[1]}
     rmse_pp = float(np.mean(rmses))
     r64 = plain["fp64"]["rmse"]
     out = {
