@@ -172,11 +172,12 @@ void launch_hyper(const HyperParams &a, cudaStream_t st);
 // First level of the statistics sum: partials (j0 + j) * kStatParts + p of job j (see misc.cu).
 constexpr int kStatParts = 64;
 // A job of at most kStatParts chunks is summed by the draw itself, without the first level.  The rule
-// looks at the job alone, so its sums do not depend on the batch it is drawn in.  K > kPairsMaxK keeps
-// the first level for every job (its rounding: see hyper_kernel).
+// looks at the job alone, so its sums do not depend on the batch it is drawn in.  Where the draw takes
+// the short chain only (K <= kHyperFastMaxK, see hyper_kernel).
+constexpr int kHyperFastMaxK = 16;
 __host__ __device__ inline bool direct_stats(int K, const HyperJob &j)
 {
-    return K <= kPairsMaxK && j.chunk1 - j.chunk0 <= kStatParts;
+    return K <= kHyperFastMaxK && j.chunk1 - j.chunk0 <= kStatParts;
 }
 void launch_stats_reduce(int K, const HyperJob *jobs, int n_jobs, int j0, const double *stats,
                          double *out, cudaStream_t st);

@@ -183,9 +183,11 @@ void launch_stats_reduce(int K, const HyperJob *jobs, int n_jobs, int j0, const 
 // The kernel is a chain of dependent FP64 operations (64 clocks each) on the path from one sweep to
 // the next: FAST shortens it where small problems wait for it (the pivots' reciprocal square roots
 // by Newton steps, reciprocals computed while the statistics load, the triangular solve by a warp).
-// K > kPairsMaxK keeps the plain operations: its draws hide the chain, and there a change of
-// rounding moves a reduced-precision chain too far (cond_pairs.cu).  K = 10, 1,000 rows, with the
-// statistics sum: 41 us, 29 us FAST.
+// K > kHyperFastMaxK keeps the plain operations: there the other half's Gram pass and draws hide
+// the chain (K = 24, 30,011 x 2,027 with a sampled noise precision: 13.5 ms for 20 sweeps plain,
+// 14.4 ms FAST, although a draw alone takes 156 and 91 us), and at K > 48 a change of rounding moves
+// a reduced-precision chain too far (cond_pairs.cu).  K = 10, 1,000 rows, with the statistics sum:
+// 41 us, 29 us FAST.
 // ------------------------------------------------------------------------------------------
 template <bool FAST>
 __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
@@ -339,17 +341,14 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
     __syncthreads();
     if (flag) goto fail;
     if constexpr (FAST) {
-        if (t < 32) {   // column by column, lane l holding v_l and v_{l + 32}
-            double v0 = t < K ? v[t] : 0.0, v1 = t + 32 < K ? v[t + 32] : 0.0;
+        if (t < 32) {   // column by column, lane l holding v_l (K <= 32)
+            double v0 = t < K ? v[t] : 0.0;
             for (int i = K - 1; i >= 0; --i) {
-                const double x = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31) * rinv[i];
-                if (t == (i & 31)) (i < 32 ? v0 : v1) = x;
+                const double x = __shfl_sync(0xffffffffu, v0, i) * rinv[i];
+                if (t == i) v0 = x;
                 if (t < i) v0 = fma(-C[i * K + t], x, v0);
-                if (t + 32 < i) v1 = fma(-C[i * K + t + 32], x, v1);
             }
-            const double sb = rsqrt_newton(bstar);
-            if (t < K) mu[t] = fma(v0, sb, mus[t]);
-            if (t + 32 < K) mu[t + 32] = fma(v1, sb, mus[t + 32]);
+            if (t < K) mu[t] = fma(v0, rsqrt_newton(bstar), mus[t]);
         }
     } else if (t == 0) {
         const double sb = rsqrt(bstar);
@@ -393,7 +392,7 @@ static void launch_hyper_t(const HyperParams &a, cudaStream_t st)
 void launch_hyper(const HyperParams &a, cudaStream_t st)
 {
     if (a.n_jobs <= 0) return;
-    if (a.K <= kPairsMaxK)
+    if (a.K <= kHyperFastMaxK)
         launch_hyper_t<true>(a, st);
     else
         launch_hyper_t<false>(a, st);

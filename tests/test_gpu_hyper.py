@@ -1,5 +1,4 @@
-"""The hyperparameter draw at the edges of its rules: a lane's one or two entries of mu (K up to 32
-and above), the short chain (K <= 48) and the plain one, and factor blocks of up to 64 statistics
+"""The hyperparameter draw at the edges of its rules: the short chain (K <= 16) and the plain one, and factor blocks of up to 64 statistics
 chunks of 64 rows, summed by the draw itself, against longer ones.  Tolerance: one transition in
 FP64, as everywhere against the oracle (1e-9 per row)."""
 import pytest
