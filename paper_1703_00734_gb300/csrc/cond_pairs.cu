@@ -424,8 +424,10 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
                     for (int u = 0; u < 4; ++u)
                         if (j0 + u <= i) assemble(M + row_off(i) + j0 + u, cur[u]);
                 }
-                bad |= !pair_vector(pr);
+                // the terms and their sum: tau g alone can leave FP32's exponents
+                const float g = Y[i].h;
                 assemble(Y + i, pr);
+                bad |= !pair_vector(pr) | !pair_vector(Y[i].h) | (Y[i].h == 0.f && g != 0.f);
             }
         }
         for (int i = active ? K + tl : tl; i < KP; i += T) {
@@ -436,11 +438,16 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
         bad |= !team.template factor<RMAX>(0);
         for (int i = tl; i < K && active; i += T) {
             const double zi = xd[i];
-            bad |= !pair_vector(zi);
             Y[i] = padd(Y[i], split(zi));
+            bad |= !pair_vector(zi) | !pair_vector(Y[i].h);
         }
         __syncwarp();
         team.back();
+        for (int i = tl; i < K; i += T) {
+            const fpair x = renorm(Y[i]);
+            bad |= !pair_vector(x.h);
+            xd[i] = join(x);
+        }
         bool ok = active;
         const bool redo = (__ballot_sync(0xffffffffu, bad) & tmask) != 0u;
         if (active && redo) {
@@ -449,8 +456,6 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
             ok = __shfl_sync(tmask, done, lane & ~(T - 1)) != 0;
             __syncwarp(tmask);
             for (int i = tl; i < K; i += T) xd[i] = reinterpret_cast<double *>(M)[NT + i];
-        } else {
-            for (int i = tl; i < K; i += T) xd[i] = join(renorm(Y[i]));
         }
         __syncwarp();
         // state, gathered copy, moment sums

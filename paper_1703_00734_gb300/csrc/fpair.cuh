@@ -95,8 +95,9 @@ __device__ __forceinline__ fpair prsqrt(fpair d)
 
 // Ranges within which a pair keeps its 48 bits through the products and sums of a conditional
 // draw, from the exponent field (infinities and NaN fall outside).  Any term below 2^70; a
-// precision's diagonal from 2^-60; a right-hand side or draw zero or from 2^-100.  Rows outside
-// take the FP64 path.
+// precision's diagonal from 2^-60; a right-hand side, a draw and the solutions of both triangular
+// solves zero or from 2^-100 (a zero that is no underflow: between right-hand side and solution lie
+// factors of at least 2^-35).  Rows outside take the FP64 path.
 __device__ __forceinline__ bool pair_below(double x)
 {
     return ((unsigned)__double2hiint(x) & 0x7fffffffu) < (1023u + 70u) << 20;
@@ -105,6 +106,11 @@ __device__ __forceinline__ bool pair_vector(double x)
 {
     const unsigned u = (unsigned)__double2hiint(x) & 0x7fffffffu;
     return u - ((1023u - 100u) << 20) < 170u << 20 || (u | (unsigned)__double2loint(x)) == 0u;
+}
+__device__ __forceinline__ bool pair_vector(float h)
+{
+    const unsigned u = __float_as_uint(h) & 0x7fffffffu;
+    return u - ((127u - 100u) << 23) < 170u << 23 || u == 0u;
 }
 __device__ __forceinline__ bool pair_diag(float h) { return h >= 0x1p-60f && h < 0x1p70f; }
 
