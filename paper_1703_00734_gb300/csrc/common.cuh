@@ -81,13 +81,11 @@ __device__ __forceinline__ bool pivot_ok(double d)
     return b >= 0x0010000000000000ll && b < 0x7ff0000000000000ll;
 }
 
-// 1 / sqrt(d) for a pivot of the FP64 Cholesky in the reduced-precision modes (FP32 or BF16
-// Gram entries, relative error ~1e-7 already); d must pass pivot_ok.  With d = m 2^E, m in
-// [1, 2) and E = 2h + p (p in {0, 1}): the FP32 unit gives 1/sqrt(m 2^p) for a float built from
-// d's top mantissa bits (relative error below 2^-21 with the truncation), widened and scaled by
-// 2^-h on the integer pipe, then one Newton step in FP64, y <- y + (y / 2)(1 - d y^2) (y / 2 by
-// the exponent too): relative error below 1e-12 with three FP64 operations and no branch.
-__device__ __forceinline__ double rsqrt_refined(double d)
+// 1 / sqrt(d) to FP32's accuracy for a d that passes pivot_ok.  With d = m 2^E, m in [1, 2) and
+// E = 2h + p (p in {0, 1}): the FP32 unit gives 1/sqrt(m 2^p) for a float built from d's top
+// mantissa bits (relative error below 2^-21 with the truncation), widened and scaled by 2^-h on
+// the integer pipe.  half: the same with a factor 1 / 2, by the exponent.
+__device__ __forceinline__ double rsqrt_seed(double d, double &half)
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(d);
     const int E = (int)(u >> 52) - 1023;
@@ -96,10 +94,31 @@ __device__ __forceinline__ double rsqrt_refined(double d)
     const uint32_t yb = __float_as_uint(rsqrtf(__uint_as_float(fb)));   // in (0.5, 1]
     const int hi = (int)(((yb & 0x7fffffffu) >> 3) + 0x38000000u);
     const int lo = (int)(yb << 29);
-    const double y = __hiloint2double(hi - h * (1 << 20), lo);
-    const double y2 = __hiloint2double(hi - (h + 1) * (1 << 20), lo);
+    half = __hiloint2double(hi - (h + 1) * (1 << 20), lo);
+    return __hiloint2double(hi - h * (1 << 20), lo);
+}
+
+// 1 / sqrt(d) for a pivot of the FP64 Cholesky in the reduced-precision modes (FP32 or BF16
+// Gram entries, relative error ~1e-7 already): one Newton step in FP64 on the seed,
+// y <- y + (y / 2)(1 - d y^2): relative error below 1e-12 with three FP64 operations and no branch.
+__device__ __forceinline__ double rsqrt_refined(double d)
+{
+    double y2;
+    const double y = rsqrt_seed(d, y2);
     const double r = fma(-(d * y), y, 1.0);
     return fma(y2, r, y);
+}
+
+// 1 / sqrt(d) to the last bit or two: the seed and one third-order step,
+// y <- y + (y / 2) r (1 + 3 r / 4) with r = 1 - d y^2 below 2^-20 (the next term is below 2^-61): five
+// FP64 operations.  0 < d, the CUDA function outside the normal range.
+__device__ __forceinline__ double rsqrt_full(double d)
+{
+    if (!pivot_ok(d)) return rsqrt(d);
+    double y2;
+    const double y = rsqrt_seed(d, y2);
+    const double r = fma(-(d * y), y, 1.0);
+    return fma(y2, r * fma(0.75, r, 1.0), y);
 }
 
 // Pivot reciprocal square root of the conditional draw: full FP64 in the FP64 mode (gathered

@@ -18,9 +18,9 @@
 // the FP32 gathers of ill-conditioned rows, to more than 2e-5 of the posterior means within ten
 // sweeps (50,000 x 12,500, K = 64, sigma 0.3: 5e-5, half of what FP32 gathers are off by).
 //
-// A row whose terms leave the range of a pair, or whose pivot loses 20 bits to cancellation (among
-// them every row that is not positive definite), is redone in FP64 by cond_row_serial, so what
-// is accepted and what is rejected is decided in FP64.
+// A row whose terms or results leave the range of a pair, or whose pivot loses 20 bits to
+// cancellation (among them every row that is not positive definite), is redone in FP64 by a
+// team, so what is accepted and what is rejected is decided in FP64.
 #include <algorithm>
 
 #include <cuda_bf16.h>
@@ -40,78 +40,12 @@ __device__ __forceinline__ float gathered<float>(double, float h) { return h; } 
 template <>
 __device__ __forceinline__ __nv_bfloat16 gathered<__nv_bfloat16>(double x, float) { return __double2bfloat16(x); }
 
-__device__ __forceinline__ float as_float(float x) { return x; }
-__device__ __forceinline__ float as_float(__nv_bfloat16 x) { return __bfloat162float(x); }
-
 __device__ __forceinline__ void decode_tri(int e, int &i, int &j)
 {
     i = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
     while (i * (i + 1) / 2 > e) --i;
     while ((i + 1) * (i + 2) / 2 <= e) ++i;
     j = e - i * (i + 1) / 2;
-}
-
-// One row in FP64 by one thread: S has room for ntri(K) + 2 K doubles; x is left at S + ntri(K).
-// False (with the error word set) if a pivot is not positive.
-template <typename GT>
-__device__ __noinline__ bool cond_row_serial(const CondParams &a, int64_t r, double *S)
-{
-    const int K = a.K, NT = ntri(K);
-    double *B = S + NT, *RI = B + K;
-    const int64_t i0 = a.item_ptr[r], i1 = a.item_ptr[r + 1];
-    const int mi = a.multi_idx[r], h = a.row_hslot[r];
-    const double tau = a.tau_row ? a.tau_row[r] : a.tau;
-    const double *hp = h >= 0 ? a.hyper + (int64_t)h * hyper_slot_len(K) : nullptr;
-    for (int e = 0, i = 0, j = 0; e < NT + K; ++e) {
-        // entry e: (i, j) of the packed lower triangle, then the right-hand side
-        double g = 0.0;
-        const int src = e < NT ? e : a.part_rhs + (e - NT);
-        if (mi >= 0) {
-            g = a.rowsum[(int64_t)mi * a.ld_sum + src];
-        } else if (mi == kFusedRow) {
-            float s = 0.f;
-            for (int64_t o = a.obs_ptr[r]; o < a.obs_ptr[r + 1]; ++o) {
-                const GT *p = static_cast<const GT *>(a.P) + (int64_t)a.obs_idx[o] * a.ldP;
-                const float u = e < NT ? as_float(p[j]) : static_cast<const float *>(a.obs_val)[o];
-                s = fmaf(as_float(p[e < NT ? i : e - NT]), u, s);
-            }
-            g = (double)s;
-        } else if (i1 > i0) {
-            g = (double)(static_cast<const float *>(a.part) + (i0 - a.item0) * (int64_t)a.ld)[src];
-        }
-        const double prior = e < NT ? (hp ? hp[K + e] : a.prior_L[(int64_t)e * a.R + r])
-                                    : (hp ? hp[K + e] : a.prior_b[(int64_t)(e - NT) * a.R + r]);
-        S[e] = fma(tau, g, prior);
-        if (++j > i) ++i, j = 0;
-    }
-    for (int j = 0; j < K; ++j) {
-        double d = S[tri(j, j)];
-        for (int k = 0; k < j; ++k) d = fma(-S[tri(j, k)], S[tri(j, k)], d);
-        if (!pivot_ok(d)) {
-            atomicOr(&a.err->flags, ERR_NOT_PD);
-            atomicMin(&a.err->first_bad_row, (int)r);
-            return false;
-        }
-        const double rs = rsqrt(d);
-        RI[j] = rs;
-        for (int i = j + 1; i < K; ++i) {
-            double s = S[tri(i, j)];
-            for (int k = 0; k < j; ++k) s = fma(-S[tri(i, k)], S[tri(j, k)], s);
-            S[tri(i, j)] = s * rs;
-        }
-    }
-    for (int i = 0; i < K; ++i) {
-        double s = B[i];
-        for (int k = 0; k < i; ++k) s = fma(-S[tri(i, k)], B[k], s);
-        B[i] = s * RI[i];
-    }
-    const double *z = a.z + (r - a.row0) * K;
-    for (int i = K - 1; i >= 0; --i) {
-        double s = B[i] + z[i];
-        for (int k = i + 1; k < K; ++k) s = fma(-S[tri(k, i)], B[k], s);
-        B[i] = s * RI[i];
-    }
-    return true;
 }
 
 // A pivot that lost 20 of its 48 bits (or is not positive, or NaN) sends its row to FP64.
@@ -340,10 +274,258 @@ struct Team {
     }
 };
 
+// What a row's Gram sums and prior are read from.
+struct RowTerms {
+    const double *ps, *pl, *pb;   // sums of several work items; prior precision and precision x mean
+    const float *pp;              // one item's sums
+    int64_t step;                 // between packed entries of the prior
+    double tau;
+    int mi;
+    bool one;
+    __device__ __forceinline__ RowTerms(const CondParams &a, int64_t r)
+    {
+        const int64_t i0 = a.item_ptr[r];
+        const int h = a.row_hslot[r];
+        mi = a.multi_idx[r];
+        one = a.item_ptr[r + 1] > i0;
+        tau = a.tau_row ? a.tau_row[r] : a.tau;
+        const double *hp = a.hyper + (int64_t)(h >= 0 ? h : 0) * hyper_slot_len(a.K) + a.K;
+        pl = h >= 0 ? hp : a.prior_L + r;
+        pb = h >= 0 ? hp + ntri(a.K) : a.prior_b + r;
+        step = h >= 0 ? 1 : a.R;
+        ps = a.rowsum + (int64_t)(mi >= 0 ? mi : 0) * a.ld_sum;
+        pp = static_cast<const float *>(a.part) + (i0 - a.item0) * (int64_t)a.ld;
+    }
+    __device__ __forceinline__ double sum(int e) const { return mi >= 0 ? ps[e] : (one ? widen(pp[e]) : 0.0); }
+};
+
+// State, gathered copy and moment sums of a drawn row (x in xd) by its team; the row's slots take the
+// old moment sums.
+template <int T, typename GT>
+__device__ __forceinline__ void store_row(const CondParams &a, int64_t r, fpair *M, fpair *Y, const double *xd, int tl)
+{
+    const int K = a.K;
+    const int64_t R = a.R;
+    if (a.keep) {
+        for (int i = tl; i < K; i += T) {
+            copy8(Y + i, a.S1 + (int64_t)i * R + r);
+            if (a.full) {
+                const double *src = a.S2 + (int64_t)tri(i, 0) * R + r;
+                fpair *dst = M + row_off(i);
+                for (int j = 0; j <= i; ++j) copy8(dst + j, src + j * R);
+            }
+        }
+    }
+    GT *g = static_cast<GT *>(a.Xg) + r * a.ldg;
+    for (int i = tl; i < K; i += T) {
+        const double xi = xd[i];
+        a.X[r * K + i] = xi;
+        g[i] = gathered<GT>(xi, (float)xi);
+    }
+    for (int i = K + tl; i < a.ldg; i += T) g[i] = gathered<GT>(0.0, 0.f);
+    if (a.keep) {
+        copies_wait();
+        for (int i = tl; i < K; i += T) {
+            const double xi = xd[i];
+            a.S1[(int64_t)i * R + r] = *reinterpret_cast<const double *>(Y + i) + xi;
+            if (a.full) {
+                double *dst = a.S2 + (int64_t)tri(i, 0) * R + r;
+                const fpair *src = M + row_off(i);
+#pragma unroll 4
+                for (int j = 0; j <= i; ++j)
+                    dst[j * R] = fma(xi, xd[j], *reinterpret_cast<const double *>(src + j));
+            }
+        }
+    }
+}
+
+// One row in FP64 by its team, x to xd.  False if a pivot is not positive.
+//
+// Four lanes (K <= 16): lane tl holds the rows tl + 4 s in registers; pivots and columns by shuffles.
+template <int RMAX, typename GT>
+__device__ __forceinline__ bool row_fp64_regs(const CondParams &a, int64_t r, fpair *M, fpair *Y, double *xd, int tl)
+{
+    constexpr int KP = 4 * RMAX;
+    constexpr unsigned kFull = 0xffffffffu;
+    const int K = a.K;
+    const RowTerms t(a, r);
+    const bool fused = t.mi == kFusedRow;
+    if (fused) {
+        Team<4, RMAX, GT> team{a, M, Y, nullptr, KP, tl, 0};
+        team.own_gram(a.obs_ptr[r], (int)(a.obs_ptr[r + 1] - a.obs_ptr[r]));   // this lane's rows
+    }
+    double m[RMAX][KP], b[RMAX], x[RMAX];
+#pragma unroll
+    for (int s = 0; s < RMAX; ++s) {
+        const int i = tl + 4 * s;
+#pragma unroll
+        for (int j = 0; j < KP; ++j)
+            if (j < 4 * s + 4)
+                m[s][j] = i < K && j <= i ? fma(t.tau, fused ? widen(M[row_off(i) + j].h) : t.sum(tri(i, j)),
+                                                t.pl[(int64_t)tri(i, j) * t.step])
+                                          : 0.0;
+        b[s] = i < K ? fma(t.tau, fused ? widen(Y[i].h) : t.sum(a.part_rhs + i), t.pb[i * t.step]) : 0.0;
+        x[s] = 0.0;
+    }
+    __syncwarp();
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < KP; ++k)
+        if (k < K) {
+            const double d = __shfl_sync(kFull, m[k / 4][k], k % 4, 4);
+            ok = ok && pivot_ok(d);
+            const double rs = ok ? rsqrt_full(d) : 0.0;
+            const double y = __shfl_sync(kFull, b[k / 4], k % 4, 4) * rs;
+            double l[RMAX];
+#pragma unroll
+            for (int s = 0; s < RMAX; ++s)
+                if (s >= k / 4) {
+                    l[s] = tl + 4 * s > k ? m[s][k] * rs : 0.0;
+                    b[s] = fma(-l[s], y, b[s]);
+                    m[s][k] = l[s];
+                }
+            if (tl == k % 4) {
+                m[k / 4][k] = rs;   // 1 / L_kk in L_kk's place
+                b[k / 4] = y;
+            }
+#pragma unroll
+            for (int j = 0; j < KP; ++j)
+                if (j > k) {
+                    const double lj = __shfl_sync(kFull, l[j / 4], j % 4, 4);
+#pragma unroll
+                    for (int s = 0; s < RMAX; ++s)
+                        if (s >= j / 4) m[s][j] = fma(-l[s], lj, m[s][j]);
+                }
+        }
+    const double *z = a.z + (r - a.row0) * K;
+#pragma unroll
+    for (int s = 0; s < RMAX; ++s)
+        if (tl + 4 * s < K) b[s] += z[tl + 4 * s];
+    // x_i from the rows below it, each lane's share of them first (x[s] is zero until known)
+#pragma unroll
+    for (int i = KP - 1; i >= 0; --i)
+        if (i < K) {
+            double v = 0.0;
+#pragma unroll
+            for (int s = 0; s < RMAX; ++s)
+                if (s >= i / 4) v = fma(m[s][i], x[s], v);
+            v += __shfl_xor_sync(kFull, v, 1);
+            v += __shfl_xor_sync(kFull, v, 2);
+            if (tl == i % 4) x[i / 4] = (b[i / 4] - v) * m[i / 4][i];
+        }
+#pragma unroll
+    for (int s = 0; s < RMAX; ++s)
+        if (tl + 4 * s < K) xd[tl + 4 * s] = x[s];
+    return ok;
+}
+
+// Wider teams: the row in the slots of its pairs (a slot is as long as a double), right-looking with the
+// right-hand side as one more row, lane tl owning the rows tl + T s.
+template <int T, int RMAX>
+__device__ __forceinline__ bool row_fp64(const CondParams &a, int64_t r, double *M, double *Y, double *xd, int tl)
+{
+    const int K = a.K;
+    const RowTerms t(a, r);
+    for (int i = tl; i < K; i += T) {
+        for (int j0 = 0; j0 <= i; j0 += 4) {
+            double g[4], p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = tri(i, min(j0 + u, i));
+                g[u] = t.sum(e);
+                p[u] = t.pl[(int64_t)e * t.step];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (j0 + u <= i) M[row_off(i) + j0 + u] = fma(t.tau, g[u], p[u]);
+        }
+        Y[i] = fma(t.tau, t.sum(a.part_rhs + i), t.pb[i * t.step]);
+    }
+    __syncwarp();
+    bool ok = true;
+    for (int k = 0, kk = 0; k < K; kk += 4 * (k >> 2) + 6, ++k) {   // kk: row_off(k)
+        const double d = M[kk + k];
+        ok = ok && pivot_ok(d);
+        const double rs = ok ? rsqrt_full(d) : 0.0, y = Y[k] * rs;
+        double l[RMAX];
+#pragma unroll
+        for (int s = 0; s < RMAX; ++s) {
+            const int i = tl + T * s;
+            l[s] = 0.0;
+            if (i > k && i < K) M[row_off(i) + k] = l[s] = M[row_off(i) + k] * rs;
+        }
+        __syncwarp();
+        if (tl == 0) M[kk + k] = rs, Y[k] = y;   // 1 / L_kk in L_kk's place
+#pragma unroll
+        for (int s = 0; s < RMAX; ++s) {
+            const int i = tl + T * s;
+            if (i > k && i < K) Y[i] = fma(-l[s], y, Y[i]);
+        }
+        for (int j = k + 1, jj = kk + 4 * (k >> 2) + 6; j < K; jj += 4 * (j >> 2) + 6, ++j) {
+            const double lj = M[jj + k];
+#pragma unroll
+            for (int s = 0; s < RMAX; ++s) {
+                const int i = tl + T * s;
+                if (i >= j && i < K) M[row_off(i) + j] = fma(-l[s], lj, M[row_off(i) + j]);
+            }
+        }
+        __syncwarp();
+    }
+    const double *z = a.z + (r - a.row0) * K;
+    for (int i = tl; i < K; i += T) Y[i] += z[i];
+    __syncwarp();
+    for (int i = K - 1; i >= 0; --i) {
+        const double *row = M + row_off(i);
+        const double x = Y[i] * row[i];
+        for (int k = tl; k < i; k += T) Y[k] = fma(-row[k], x, Y[k]);
+        if (tl == 0) xd[i] = x;
+        __syncwarp();
+    }
+    return ok;
+}
+
+// The rows row0 + (set bits of `rows`) of this CUDA block in FP64, a team each: those that pairs cannot
+// hold, after the block's other rows.  They are dealt out anew, so that the teams of a warp (whose
+// FP64 instructions cost the same whatever the active lanes) have one each, and stand apart from the
+// pair draw, whose registers they would cost.  A lane alone on a row, where its team found it, waited
+// on K^3 / 6 dependent operations: 60,000 rows of K / 2 observations and 20,000 ordinary ones, sigma =
+// 0.002 to 0.003, where most rows lose their pivots' bits, us a sweep with FP64 teams or threads for
+// all rows / pairs and a lane / pairs and these: K = 10 247 / 431 / 276, K = 16 487 / 2,035 / 594,
+// K = 24 1,830 / 4,350 / 1,559 (ordinary noise: 250 / 185, 489 / 279, 1,744 / 677).
+template <int T, int RMAX, typename GT>
+__device__ __noinline__ void redo_rows(const CondParams &a, int64_t row0, unsigned long long rows, fpair *M, fpair *Y,
+                                       double *xd, int tm, int tl, int n_teams)
+{
+    const int n = __popcll(rows);
+    for (int base = 0; base < n; base += n_teams) {
+        const bool mine = base + tm < n;
+        if (!__any_sync(0xffffffffu, mine)) break;
+        unsigned long long left = rows;      // teams without a row repeat the last one and drop it
+        for (int q = min(base + tm, n - 1); q > 0; --q) left &= left - 1;
+        const int64_t r = row0 + __ffsll((long long)left) - 1;
+        __syncwarp();
+        bool ok;
+        if constexpr (T == 4)
+            ok = row_fp64_regs<RMAX, GT>(a, r, M, Y, xd, tl);
+        else
+            ok = row_fp64<T, RMAX>(a, r, reinterpret_cast<double *>(M), reinterpret_cast<double *>(Y), xd, tl);
+        __syncwarp();
+        if (mine && ok) store_row<T, GT>(a, r, M, Y, xd, tl);
+        if (mine && !ok && tl == 0) {
+            atomicOr(&a.err->flags, ERR_NOT_PD);
+            atomicMin(&a.err->first_bad_row, (int)r);
+        }
+        __syncwarp();
+    }
+}
+
 template <int T, int RMAX, typename GT>
 __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__ CondParams a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ unsigned long long redo_rest;   // rows of the block left for FP64
+    if (threadIdx.x == 0) redo_rest = 0ull;
+    __syncthreads();
     const int K = a.K, NT = ntri(K), KP = padded4(K);
     const int lane = threadIdx.x & 31, tl = threadIdx.x % T, tm = threadIdx.x / T;
     const int n_teams = blockDim.x / T;
@@ -448,52 +630,14 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
             bad |= !pair_vector(x.h);
             xd[i] = join(x);
         }
-        bool ok = active;
         const bool redo = (__ballot_sync(0xffffffffu, bad) & tmask) != 0u;
-        if (active && redo) {
-            int done = 0;
-            if (tl == 0) done = cond_row_serial<GT>(a, r, reinterpret_cast<double *>(M)) ? 1 : 0;
-            ok = __shfl_sync(tmask, done, lane & ~(T - 1)) != 0;
-            __syncwarp(tmask);
-            for (int i = tl; i < K; i += T) xd[i] = reinterpret_cast<double *>(M)[NT + i];
-        }
         __syncwarp();
-        // state, gathered copy, moment sums
-        if (ok) {
-            if (a.keep) {
-                for (int i = tl; i < K; i += T) {
-                    copy8(Y + i, a.S1 + (int64_t)i * R + r);
-                    if (a.full) {
-                        const double *src = a.S2 + (int64_t)tri(i, 0) * R + r;
-                        fpair *dst = M + row_off(i);
-                        for (int j = 0; j <= i; ++j) copy8(dst + j, src + j * R);
-                    }
-                }
-            }
-            GT *g = static_cast<GT *>(a.Xg) + r * a.ldg;
-            for (int i = tl; i < K; i += T) {
-                const double xi = xd[i];
-                a.X[r * K + i] = xi;
-                g[i] = gathered<GT>(xi, (float)xi);
-            }
-            for (int i = K + tl; i < a.ldg; i += T) g[i] = gathered<GT>(0.0, 0.f);
-            if (a.keep) {
-                copies_wait();
-                for (int i = tl; i < K; i += T) {
-                    const double xi = xd[i];
-                    a.S1[(int64_t)i * R + r] = *reinterpret_cast<const double *>(Y + i) + xi;
-                    if (a.full) {
-                        double *dst = a.S2 + (int64_t)tri(i, 0) * R + r;
-                        const fpair *src = M + row_off(i);
-#pragma unroll 4
-                        for (int j = 0; j <= i; ++j)
-                            dst[j * R] = fma(xi, xd[j], *reinterpret_cast<const double *>(src + j));
-                    }
-                }
-            }
-        }
+        if (active && !redo) store_row<T, GT>(a, r, M, Y, xd, tl);
+        if (active && redo && tl == 0) atomicOr(&redo_rest, 1ull << q);
         __syncwarp();
     }
+    __syncthreads();
+    if (redo_rest != 0ull) redo_rows<T, RMAX, GT>(a, blk.row0, redo_rest, M, Y, xd, tm, tl, n_teams);
     // per-block statistics of the new state for the next hyperparameter draw (only blocks whose
     // factor draws its hyperparameters: every row of a block shares its subset's prior), read back
     // from the state rows this block has just written, each entry over the rows in order

@@ -93,16 +93,6 @@ void launch_stats(int K, const StatChunk *chunks, int n_chunks, const double *X,
 // Block-level dense FP64 linear algebra on K x K row-major matrices in shared memory.
 // ------------------------------------------------------------------------------------------
 
-// 1 / sqrt(d) to the last bit or two: the FP32 reciprocal square root and two Newton steps in FP64
-// (rsqrt_refined is the first), seven dependent FP64 operations; 0 < d, the CUDA function outside
-// the normal range.
-__device__ __forceinline__ double rsqrt_newton(double d)
-{
-    if (!pivot_ok(d)) return rsqrt(d);
-    const double y = rsqrt_refined(d);
-    return fma(0.5 * y, fma(-(d * y), y, 1.0), y);
-}
-
 // In-place lower Cholesky (right-looking); rinv[k] = 1 / L_kk.  Returns false (uniformly) if a
 // pivot is not > 0.  Two barriers per column: the trailing update of column k uses the unscaled
 // column times 1 / d_k, and column k is scaled during the next pivot step.
@@ -116,7 +106,7 @@ __device__ bool block_chol(double *A, int K, double *rinv, int *flag)
             if (!(d > 0.0)) {
                 *flag = 1;
             } else {
-                const double r = FAST ? rsqrt_newton(d) : rsqrt(d);
+                const double r = FAST ? rsqrt_full(d) : rsqrt(d);
                 A[k * K + k] = d * r;
                 rinv[k] = r;
             }
@@ -182,7 +172,7 @@ void launch_stats_reduce(int K, const HyperJob *jobs, int n_jobs, int j0, const 
 //
 // The kernel is a chain of dependent FP64 operations (64 clocks each) on the path from one sweep to
 // the next: FAST shortens it where small problems wait for it (the pivots' reciprocal square roots
-// by Newton steps, reciprocals computed while the statistics load, the triangular solve by a warp).
+// from FP32 ones, reciprocals computed while the statistics load, the triangular solve by a warp).
 // K > kHyperFastMaxK keeps the plain operations: there the other half's Gram pass and draws hide
 // the chain (K = 24, 30,011 x 2,027 with a sampled noise precision: 13.5 ms for 20 sweeps plain,
 // 14.4 ms FAST, although a draw alone takes 156 and 91 us), and at K > 48 a change of rounding moves
@@ -348,7 +338,7 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
                 if (t == i) v0 = x;
                 if (t < i) v0 = fma(-C[i * K + t], x, v0);
             }
-            if (t < K) mu[t] = fma(v0, rsqrt_newton(bstar), mus[t]);
+            if (t < K) mu[t] = fma(v0, rsqrt_full(bstar), mus[t]);
         }
     } else if (t == 0) {
         const double sb = rsqrt(bstar);
