@@ -18,6 +18,14 @@
 // the FP32 gathers of ill-conditioned rows, to more than 2e-5 of the posterior means within ten
 // sweeps (50,000 x 12,500, K = 64, sigma 0.3: 5e-5, half of what FP32 gathers are off by).
 //
+// Pairs stand in for FP64 only where the Gram sums' own rounding is what a row's draw is off by.  A
+// row whose sums make up less than 2^-16 of every diagonal entry (above all a row without
+// observations, which is its prior and its normals) is drawn in FP64.  Median error of a draw against
+// 64-bit arithmetic on 64-bit partners at K = 16 with priors of condition 1e4, FP64 with its refined
+// pivots for all rows / pairs for all rows / this: rows without observations 2.5e-13 / 1.4e-12 /
+// 3.8e-14; with 1 to 15 observations 1.08e-7 (FP32) and 1.36e-3 (BF16), with 16 to 400 6.0e-8 and
+// 4.6e-4, all three alike to three digits, as for K = 9 to 48.
+//
 // A row whose terms or results leave the range of a pair, or whose pivot loses 20 bits to
 // cancellation (among them every row that is not positive definite), is redone in FP64 by a
 // team, so what is accepted and what is rejected is decided in FP64.
@@ -50,6 +58,9 @@ __device__ __forceinline__ void decode_tri(int e, int &i, int &j)
 
 // A pivot that lost 20 of its 48 bits (or is not positive, or NaN) sends its row to FP64.
 constexpr float kPivotLoss = 0x1p-20f;
+// The part of some diagonal entry that a row's sums must make up: their own rounding, 2^-24 of them, is
+// then at least 2^-40 of the entry, 16 times a pair operation's 2^-44.
+constexpr float kSumsShare = 0x1p-16f;
 
 }  // namespace
 
@@ -540,7 +551,7 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
         const int q = q0 + tm;
         const bool active = q < q_end;
         const int64_t r = blk.row0 + (active ? q : 0);
-        bool bad = false;
+        bool bad = false, sums = false;
         // G, r and the prior (teams past the block's rows carry an identity)
         if (active) {
             const int64_t i0 = a.item_ptr[r], i1 = a.item_ptr[r + 1];
@@ -594,6 +605,7 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
             for (int u = 0; u < 4; ++u) nxt[u] = tl < K ? pl[(int64_t)tri(tl, min(u, tl)) * step] : 0.0;
             for (int i = tl; i < K; i += T) {
                 const double pr = pb[i * step];
+                const float gd = M[row_off(i) + i].h;
                 for (int j0 = 0; j0 <= i; j0 += 4) {
                     double cur[4];
 #pragma unroll
@@ -606,6 +618,7 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
                     for (int u = 0; u < 4; ++u)
                         if (j0 + u <= i) assemble(M + row_off(i) + j0 + u, cur[u]);
                 }
+                sums |= tau.h * gd >= kSumsShare * M[row_off(i) + i].h;
                 // the terms and their sum: tau g alone can leave FP32's exponents
                 const float g = Y[i].h;
                 assemble(Y + i, pr);
@@ -617,20 +630,25 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
             Y[i] = fpair{0.f, 0.f};
         }
         __syncwarp();
-        bad |= !team.template factor<RMAX>(0);
-        for (int i = tl; i < K && active; i += T) {
-            const double zi = xd[i];
-            Y[i] = padd(Y[i], split(zi));
-            bad |= !pair_vector(zi) | !pair_vector(Y[i].h);
+        const unsigned out = __ballot_sync(0xffffffffu, bad) & tmask, in = __ballot_sync(0xffffffffu, sums) & tmask;
+        bool redo = out != 0u || in == 0u;
+        if (__any_sync(0xffffffffu, active && !redo)) {
+            bad |= !team.template factor<RMAX>(0);
+            for (int i = tl; i < K && active; i += T) {
+                const double zi = xd[i];
+                Y[i] = padd(Y[i], split(zi));
+                bad |= !pair_vector(zi) | !pair_vector(Y[i].h);
+            }
+            __syncwarp();
+            team.back();
+            for (int i = tl; i < K; i += T) {
+                const fpair x = renorm(Y[i]);
+                bad |= !pair_vector(x.h);
+                xd[i] = join(x);
+            }
         }
-        __syncwarp();
-        team.back();
-        for (int i = tl; i < K; i += T) {
-            const fpair x = renorm(Y[i]);
-            bad |= !pair_vector(x.h);
-            xd[i] = join(x);
-        }
-        const bool redo = (__ballot_sync(0xffffffffu, bad) & tmask) != 0u;
+        const unsigned lost = __ballot_sync(0xffffffffu, bad) & tmask;
+        redo = redo || lost != 0u;
         __syncwarp();
         if (active && !redo) store_row<T, GT>(a, r, M, Y, xd, tl);
         if (active && redo && tl == 0) atomicOr(&redo_rest, 1ull << q);

@@ -68,6 +68,23 @@ def test_pivots_that_lose_more_are_fp64s(K, prec):
     assert (err[~lossy] <= 4 * K * 2.0 ** -44).all()
 
 
+@pytest.mark.parametrize("K", KS)
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_rows_whose_terms_are_fp64s(K, prec):
+    """Rows without observations, and rows whose sums are below 2^-16 of their prior in every diagonal
+    entry (2^-32 9 48 here): the prior and the draw are FP64's and so is x.  Diagonal priors: about
+    eight roundings an entry, here and in the reference, so 2^-49."""
+    rng = np.random.default_rng(K)
+    n = rng.integers(1, K, D)
+    n[::3] = 0
+    diag = rng.uniform(1.0, 2.0, (D, K))
+    diag[1::3] *= 2.0 ** 32
+    err, kappa = _draw(K, 1.0, n, prec, (rng.standard_normal((D, K)), diag[:, :, None] * np.eye(K)))
+    own = np.arange(D) % 3 < 2
+    assert (err[own] <= 2.0 ** -49).all(), np.sort(err[own])[-5:] * 2.0 ** 49
+    assert (err[~own] <= 4 * K * 2.0 ** -44 * kappa[~own]).all()
+
+
 @pytest.mark.parametrize("K", [16, 24])
 def test_low_noise_rows_stay_near_the_speed_of_the_others(K):
     """K / 2 observations a row: at sigma = 2e-3 nearly every row loses its pivots' bits, at 0.5 none.
