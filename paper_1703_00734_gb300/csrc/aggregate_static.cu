@@ -186,9 +186,9 @@ cudaError_t launch_rounds(int K, int64_t R, int64_t J, const double *mu, const d
     blocks(bmf::ntri(K) + 3 * K, re, se);
     blocks(bmf::ntri(K) + 2 * K, rs, ss);
     cudaError_t e = cudaSuccess;
-    if (sp > 48 * 1024) e = cudaFuncSetAttribute(static_pd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp);
-    if (!e && se > 48 * 1024) e = cudaFuncSetAttribute(static_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)se);
-    if (!e && ss > 48 * 1024) e = cudaFuncSetAttribute(static_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
+    e = bmf::allow_smem(static_pd_kernel, sp);
+    if (!e) e = bmf::allow_smem(static_eig_kernel, se);
+    if (!e) e = bmf::allow_smem(static_solve_kernel, ss);
     if (e) return e;
     Round w;
     w.ncorr = reinterpret_cast<unsigned long long *>(scr);

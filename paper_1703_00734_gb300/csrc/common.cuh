@@ -11,6 +11,20 @@ namespace bmf {
 
 constexpr int kWarp = 32;
 
+// Lets a kernel take more than the default 48 KB of dynamic shared memory: always the same size, the
+// most it ever takes or more, whatever this launch takes.  The limit belongs to the kernel on its
+// device, not to a context: a launch that set its own size could lower what another host thread has
+// just set for a larger launch of its own, which would then be refused.  227 KB is what a block can
+// have; the kernels' static arrays, where they have any, are below 1 KB.
+constexpr size_t kSmemBlock = 227 * 1024, kSmemMost = kSmemBlock - 1024;
+template <typename F>
+inline cudaError_t allow_smem(F *kernel, size_t bytes, size_t most = kSmemMost)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Packed lower-triangular index of (i, j), i >= j, row by row.
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 __host__ __device__ constexpr int ntri(int K) { return K * (K + 1) / 2; }

@@ -333,9 +333,7 @@ static void launch_cond_t(const CondParams &a, int n_blocks, cudaStream_t st)
 {
     if (launch_cond_fixed<GT, AT>(a, n_blocks, st)) return;
     const size_t smem = (size_t)cond_slots(a.K) * kCondStride * sizeof(double);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(cond_kernel<GT, AT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    allow_smem(cond_kernel<GT, AT>, smem);
     cond_kernel<GT, AT><<<n_blocks, kCondBlock, smem, st>>>(a);
 }
 

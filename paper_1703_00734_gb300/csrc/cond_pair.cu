@@ -328,9 +328,7 @@ template <int K>
 static void launch_pair_k(const CondParams &a, int n_blocks, cudaStream_t st)
 {
     const int smem = a.keep ? cond_pair_smem(K) : 0;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(cond_pair_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             cond_pair_smem(K));
+    allow_smem(cond_pair_kernel<K>, smem);
     cond_pair_kernel<K><<<n_blocks, kPairThreads, smem, st>>>(a);
 }
 

@@ -694,8 +694,7 @@ static void launch_team_t(const CondParams &a, int n_blocks, int sms, cudaStream
     if (threads == 64)
         while (parts < kCondBlock / teams && (int64_t)n_blocks * parts < (int64_t)8 * sms * fit(threads)) parts *= 2;
     const size_t smem = bytes(threads);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(cond_pairs_kernel<T, RMAX, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(cond_pairs_kernel<T, RMAX, GT>, smem);
     cond_pairs_kernel<T, RMAX, GT><<<dim3(n_blocks, parts), threads, smem, st>>>(a);
 }
 

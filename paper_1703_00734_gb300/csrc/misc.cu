@@ -374,8 +374,7 @@ template <bool FAST>
 static void launch_hyper_t(const HyperParams &a, cudaStream_t st)
 {
     const size_t smem = (size_t)(4 * a.K * a.K + 6 * a.K + 256) * sizeof(double);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(hyper_kernel<FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(hyper_kernel<FAST>, smem);
     hyper_kernel<FAST><<<a.n_jobs, 256, smem, st>>>(a);
 }
 
@@ -558,8 +557,7 @@ void launch_mm(const MMParams &a, cudaStream_t st)
     const size_t per_row = (size_t)(ntri(a.K) + 2 * a.K);
     const int rb = row_block(per_row);
     const size_t smem = per_row * rb * sizeof(double);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(mm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(mm_kernel, smem);
     mm_kernel<<<(int)((n + rb - 1) / rb), rb, smem, st>>>(a);
 }
 
@@ -735,25 +733,19 @@ void launch_aggregate(const AggParams &a, cudaStream_t st)
             const size_t per = agg_pd_slots(a.K);
             const int rb = row_block_small(per);
             const size_t smem = per * rb * sizeof(double);
-            if (smem > 48 * 1024)
-                cudaFuncSetAttribute(aggregate_pd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
+            allow_smem(aggregate_pd_kernel, smem);
             aggregate_pd_kernel<<<(int)((n_pairs + rb - 1) / rb), rb, smem, st>>>(a, n_pairs);
         }
         const size_t per = agg_corr_slots(a.K);
         const int rb = row_block_small(per);
         const size_t smem = per * rb * sizeof(double);
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(aggregate_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+        allow_smem(aggregate_eig_kernel, smem);
         aggregate_eig_kernel<<<(int)((n_pairs + rb - 1) / rb), rb, smem, st>>>(a);
     }
     const size_t per = agg_slots(a.K);
     const int rb = row_block_small(per);
     const size_t smem = per * rb * sizeof(double);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(aggregate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    allow_smem(aggregate_kernel, smem);
     aggregate_kernel<<<(int)((a.n_rows + rb - 1) / rb), rb, smem, st>>>(a);
 }
 

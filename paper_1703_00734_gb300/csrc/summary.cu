@@ -504,10 +504,8 @@ cudaError_t launch_summary(const SummaryParams &p, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     // samples too many for the FP32 copies to fit beside them: every row takes the second form
     const bool fast = smem <= 200 * 1024;
-    if (fast && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && smem_all > 48 * 1024)
-        e = cudaFuncSetAttribute(cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_all);
+    if (fast) e = allow_smem(cluster_kernel<true>, smem);
+    if (e == cudaSuccess) e = allow_smem(cluster_kernel<false>, smem_all, kSmemBlock);   // (no static arrays)
     if (e == cudaSuccess) e = cudaMemsetAsync(p.over_n, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     if (fast)
@@ -518,8 +516,7 @@ cudaError_t launch_summary(const SummaryParams &p, cudaStream_t st)
     const size_t per = 2 * (size_t)ntri(p.K) + 2 * p.K;
     const int rb = row_block(per);
     const size_t fit = per * rb * sizeof(double);
-    if (fit > 48 * 1024)
-        e = cudaFuncSetAttribute(fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fit);
+    e = allow_smem(fit_kernel, fit);
     if (e != cudaSuccess) return e;
     fit_kernel<<<(unsigned)((p.n_rows + rb - 1) / rb), rb, fit, st>>>(p);
     return cudaGetLastError();

@@ -414,9 +414,7 @@ template <int KT, bool SPLIT>
 static void launch_tf32_t(const GramParams &a, int grid, cudaStream_t st)
 {
     const size_t smem = (size_t)4 * kWideObs * (KT + 8) * 4;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(gram_wide_tf32<KT, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    allow_smem(gram_wide_tf32<KT, SPLIT>, smem);
     gram_wide_tf32<KT, SPLIT><<<grid, 128, smem, st>>>(a);
 }
 
@@ -440,16 +438,13 @@ void launch_gram_wide(int K, int prec, const GramParams &a, int grid, cudaStream
         const size_t smem = (size_t)4 * kWideObs * (K + 1) * 8;
         const int nv = ntri(K) + K;
         if (nv <= 18 * 32) {
-            if (smem > 48 * 1024)
-                cudaFuncSetAttribute(gram_wide_fp64<18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_smem(gram_wide_fp64<18>, smem);
             gram_wide_fp64<18><<<grid, 128, smem, st>>>(a);
         } else if (nv <= 38 * 32) {
-            if (smem > 48 * 1024)
-                cudaFuncSetAttribute(gram_wide_fp64<38>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_smem(gram_wide_fp64<38>, smem);
             gram_wide_fp64<38><<<grid, 128, smem, st>>>(a);
         } else {
-            if (smem > 48 * 1024)
-                cudaFuncSetAttribute(gram_wide_fp64<67>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_smem(gram_wide_fp64<67>, smem);
             gram_wide_fp64<67><<<grid, 128, smem, st>>>(a);
         }
         return;
@@ -725,8 +720,7 @@ static void launch_cond_team_t(const CondParams &a, int n_blocks, int sms, cudaS
     const int per_sm = (int)std::max<size_t>(1, (size_t)220 * 1024 / smem);
     int parts = 1;
     while (parts < kCondBlock / NTEAM && (int64_t)n_blocks * parts < (int64_t)8 * sms * per_sm) parts *= 2;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(cond_team_kernel<GT, AT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(cond_team_kernel<GT, AT, T>, smem);
     cond_team_kernel<GT, AT, T><<<dim3(n_blocks, parts), 32 * kWideWarps, smem, st>>>(a);
 }
 
