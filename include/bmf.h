@@ -91,8 +91,9 @@
  *      fail the call with BMF_E_CUDA (probability below 1e-80);
  *    kind 4, noise chi-square variate k of a subset (factor W): drawn the same way with the
  *      dof of the layout above.
- *  The numbers depend only on (seed, subset, factor, t, position): batching a stage or
- *  splitting sweeps across calls does not change them.  bmf_generate_draws returns them.
+ *  The numbers depend only on (seed, subset, factor, t, position) and, in the rounding of the
+ *  last bits, on whether K is above 48: batching a stage, splitting sweeps across calls or
+ *  another precision mode does not change them.  bmf_generate_draws returns them.
  *
  * Memory and errors.  The context owns all device memory it allocates.  Host pointers passed
  * in are read during the call only; the caller keeps ownership.  Every call is synchronous

@@ -1710,10 +1710,12 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
     c->rmse_part = c->mem.alloc<double>(2 * c->rmse_blocks);
     c->rmse_out = c->mem.alloc<double>(2);
     c->err_d = c->mem.alloc<DevError>(1);
-    // the normals' tables, except where reduced-precision gathers meet K > kPairsMaxK: rounding the
-    // draws differently there moves a chain by half of what its FP32 gathers are off by (see
-    // cond_pairs.cu), so they keep the FP64 functions
-    if (c->prec == BMF_FP64 || K <= kPairsMaxK) c->gen_tab = c->mem.alloc<GenTables>(1);
+    // the normals' tables up to K = 48, the FP64 functions above, in every precision mode: a context's
+    // numbers are the same in all of them.  Rounding the normals the other way moves the posterior
+    // means of ten FP32 sweeps (20,000 x 5,000, 62 entries a row, sigma = 0.3) by 8e-7 at K = 40, 5e-7
+    // at K = 48, 9e-6 at K = 60 and 6e-5 at K = 64 (BF16: 4e-14, FP64: 2e-13), where the FP32 gathers
+    // themselves are off by 1e-4; above K = 48 the generator's time is hidden beside the draws
+    if (K <= kPairsMaxK) c->gen_tab = c->mem.alloc<GenTables>(1);
     c->aggX = c->mem.alloc<double>(N * K);
     c->aggW = c->mem.alloc<double>(D * K);
     c->ncorr_d = c->mem.alloc<unsigned long long>(1);

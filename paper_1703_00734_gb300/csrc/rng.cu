@@ -4,7 +4,9 @@
 // as 1, 2, 3", SC'11) with key (seed, 0) and counter (index, t, tag, attempt), t the 1-based
 // sweep number of the subset's chain and tag = subset id * 256 + factor * 16 + kind.  Every
 // number is a pure function of its position, so the draws do not depend on batching, on the
-// launch shape or on how sweeps are split across calls.
+// launch shape, on the precision mode or on how sweeps are split across calls.  (Their last bits
+// depend on the form of the normals, which K alone chooses: tables up to K = 48, the FP64
+// functions above.)
 //   kind 2 (hyperparameter normals) and kind 3 (z of the rows): element e of the stream comes
 //     from call e / 4; words (0, 1) give elements 4q, 4q + 1 and words (2, 3) elements
 //     4q + 2, 4q + 3 by Box-Muller (cosine, sine), u1 = (top 53 bits + 1) 2^-53 in (0, 1] and
@@ -89,7 +91,7 @@ __device__ __forceinline__ double sqrt_unit(double t)
     return hi == 0 ? 0.0 : s;
 }
 
-// The same with the FP64 functions (rounded differently in the last bit).
+// The same with the FP64 functions (rounded differently in the last bits), for K > 48.
 __device__ __forceinline__ void box_muller_fp64(uint64_t a, uint64_t b, double &z0, double &z1)
 {
     const double r = sqrt(-2.0 * log(u_open0(a)));
