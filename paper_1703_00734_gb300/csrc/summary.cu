@@ -94,7 +94,7 @@ size_t cluster_smem(int K, int S, int cap, bool fast)
 }  // namespace
 
 // lambda-means of one row per warp and the covariances of its chosen clusters.  FAST rows keep at
-// most kFastCentres clusters; rows that open more are listed for a second launch with room for
+// most `cap` clusters; rows that open more are listed for a second launch with room for
 // every sample's own (2 S + 1 within a round: a centre opened in the round is its sample).
 //
 // The distances decide only comparisons (which centre is nearest, whether it is beyond lambda):
@@ -504,15 +504,31 @@ cudaError_t launch_summary(const SummaryParams &p, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     // samples too many for the FP32 copies to fit beside them: every row takes the second form
     const bool fast = smem <= 200 * 1024;
-    if (fast) e = allow_smem(cluster_kernel<true>, smem);
-    if (e == cudaSuccess) e = allow_smem(cluster_kernel<false>, smem_all, kSmemBlock);   // (no static arrays)
+    // the second in FP32 distances too where the copies of samples and as many centres fit
+    const size_t smem_wide = cluster_smem(p.K, p.S, all, true);
+    const bool wide = fast && smem_wide <= kSmemBlock;
+    if (fast) e = allow_smem(cluster_kernel<true>, std::max(smem, wide ? smem_wide : 0), kSmemBlock);   // (no static arrays)
+    if (e == cudaSuccess) e = allow_smem(cluster_kernel<false>, smem_all, kSmemBlock);
     if (e == cudaSuccess) e = cudaMemsetAsync(p.over_n, 0, sizeof(int32_t), st);
+    int dev = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (fast)
+    // how many rows are listed is not known here: as many warps as fit on the GPU step through the list.
+    // 20,000 rows of 200 samples at K = 10 that all open 200, 60 or 40 clusters: 134.7, 52.2, 38.6 ms with
+    // a warp each in FP64; 256, 118, 85 ms with two warps per SM after the first launch; 34, 16, 13 ms now
+    auto warps = [&](size_t bytes) {
+        return (unsigned)std::min<int64_t>(p.n_rows, (int64_t)sms * std::min<size_t>(32, kSmemBlock / (bytes + 1024) + 1));
+    };
+    if (fast) {
         cluster_kernel<true><<<(unsigned)p.n_rows, 32, smem, st>>>(p, cap, nullptr, nullptr, p.over, p.over_n);
-    if (!fast || p.mode != 0)
-        cluster_kernel<false><<<(unsigned)std::min<int64_t>(p.n_rows, fast ? 304 : p.n_rows), 32, smem_all, st>>>(
-            p, all, fast ? p.over : nullptr, fast ? p.over_n : nullptr, nullptr, nullptr);
+        if (p.mode != 0 && wide)
+            cluster_kernel<true><<<warps(smem_wide), 32, smem_wide, st>>>(p, all, p.over, p.over_n, nullptr, nullptr);
+        else if (p.mode != 0)
+            cluster_kernel<false><<<warps(smem_all), 32, smem_all, st>>>(p, all, p.over, p.over_n, nullptr, nullptr);
+    } else {
+        cluster_kernel<false><<<(unsigned)p.n_rows, 32, smem_all, st>>>(p, all, nullptr, nullptr, nullptr, nullptr);
+    }
     const size_t per = 2 * (size_t)ntri(p.K) + 2 * p.K;
     const int rb = row_block(per);
     const size_t fit = per * rb * sizeof(double);
