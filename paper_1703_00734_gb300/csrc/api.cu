@@ -65,6 +65,9 @@ struct Side {
     std::vector<CondBlock> h_blocks;
     std::vector<int64_t> slot_blk;    // [S+1] first block of each slot
     CondBlock *blocks = nullptr;
+    int32_t *bare = nullptr;          // rows without observations, in order (float-pair draws)
+    std::vector<int64_t> h_bare_ptr;  // [blocks+1] first of them of each block
+    double *bare_factor = nullptr;    // [ntri(K) + K][them], formed by each call
     StatChunk *chunks = nullptr;      // the same row ranges, for the standalone statistics pass
     int64_t stat0 = 0;                // first statistics slot of this arena
     int32_t *multi_idx = nullptr;     // [R] slot in rowsum or -1
@@ -90,13 +93,13 @@ constexpr int kCopyGroups = 16;   // copy groups of a host draw buffer (events p
 struct bmf_ctx {
     ~bmf_ctx()
     {
-        for (cudaStream_t x : {st2, st3, st4, st5, cap})
+        for (cudaStream_t x : {st2, st3, st4, st5, st6, cap})
             if (x) {
                 cudaStreamSynchronize(x);
                 cudaStreamDestroy(x);
             }
         for (cudaEvent_t e : {ev_fork, ev_fac[0], ev_fac[1], ev_hyp[0], ev_hyp[1], ev_cdone, ev_tail,
-                              ev_tail2, ev_rmse, ev_gen[0], ev_gen[1]})
+                              ev_tail2, ev_rmse, ev_gen[0], ev_gen[1], ev_bare[0], ev_bare[1]})
             if (e) cudaEventDestroy(e);
         for (cudaEvent_t e : ev_copyq)
             if (e) cudaEventDestroy(e);
@@ -117,10 +120,11 @@ struct bmf_ctx {
     cudaStream_t st3 = nullptr;      // conditional stream of the chunked schedule
     cudaStream_t st4 = nullptr;      // tail stream: test RMSE
     cudaStream_t st5 = nullptr;      // generator stream: the draws of the sweep after next
+    cudaStream_t st6 = nullptr;      // FP64 draws of rows without observations, beside the float pairs
     cudaStream_t cap = nullptr;      // capture stream of the graph schedule (the context stream
                                      // may be the legacy default stream, which cannot capture)
     cudaEvent_t ev_fork = nullptr, ev_fac[2] = {nullptr, nullptr}, ev_hyp[2] = {nullptr, nullptr};
-    cudaEvent_t ev_chunk[kMaxChunks] = {}, ev_cdone = nullptr;
+    cudaEvent_t ev_chunk[kMaxChunks] = {}, ev_cdone = nullptr, ev_bare[2] = {nullptr, nullptr};
     cudaEvent_t ev_tail = nullptr, ev_tail2 = nullptr, ev_rmse = nullptr, ev_gen[2] = {nullptr, nullptr};
     // a host draw buffer is copied on the generator stream in groups of sweeps, an event after
     // each group, so that sweep t waits only for its own group
@@ -404,6 +408,7 @@ bmf_status check_dev_error(bmf_ctx *c)
     if (c->st3) CUDA_TRY(c, cudaStreamSynchronize(c->st3));
     if (c->st4) CUDA_TRY(c, cudaStreamSynchronize(c->st4));
     if (c->st5) CUDA_TRY(c, cudaStreamSynchronize(c->st5));
+    if (c->st6) CUDA_TRY(c, cudaStreamSynchronize(c->st6));
     DevError h;
     CUDA_TRY(c, cudaMemcpyAsync(&h, c->err_d, sizeof(h), cudaMemcpyDeviceToHost, c->st));
     CUDA_TRY(c, cudaStreamSynchronize(c->st));
@@ -1053,6 +1058,9 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             cp.S2 = me.S2;
             cp.stats = c->stats;
             cp.parts_done = c->parts_done;
+            // rows without observations in FP64 beside the float pairs, where a factor carries priors of
+            // its rows' own (the others' statistics wait for all rows of a block)
+            cp.bare_apart = me.bare != nullptr && nj[f] < sl1 - sl0 ? 1 : 0;
             cp.err = c->err_d;
             cp.obs_ptr = me.ptr;
             cp.obs_idx = me.idx;
@@ -1063,12 +1071,28 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
             const int team = K >= kTeamMinK
                                  ? (c->sched.cond_lanes > 0 ? c->sched.cond_lanes : cond_team_size(K))
                                  : 1;
+            cudaError_t bare_err = cudaSuccess;
             auto cond_chunk = [&](int64_t ba, int64_t bb, cudaStream_t sx) {
                 if (bb <= ba) return;
                 CondParams q = cp;
                 q.blocks = me.blocks + ba;
                 q.blk0 = me.stat0 + ba;
-                traced(c, sx, f == 0 ? K_COND_X : K_COND_W, 1, [&] {
+                const BareRows w{me.bare, me.bare_factor, me.h_bare_ptr.back(), me.h_bare_ptr[ba], me.h_bare_ptr[bb]};
+                const bool bare = cp.bare_apart && w.last > w.first;
+                // their priors change within a call only where a mixture's component is chosen anew
+                const bool refactor = it == 0 || any_mix[f];
+                traced(c, sx, f == 0 ? K_COND_X : K_COND_W, bare ? (refactor ? 3 : 2) : 1, [&] {
+                    if (bare) {
+                        bare_err = cudaEventRecord(c->ev_bare[0], sx);
+                        if (!bare_err) bare_err = cudaStreamWaitEvent(c->st6, c->ev_bare[0], 0);
+                        if (bare_err) return;
+                        if (refactor) launch_bare_factor(q, w, c->sms, c->st6);
+                        launch_bare_draw(c->prec, q, w, c->st6);
+                        bare_err = cudaEventRecord(c->ev_bare[1], c->st6);
+                        launch_cond_pairs(c->prec, q, (int)(bb - ba), c->sms, sx);
+                        if (!bare_err) bare_err = cudaStreamWaitEvent(sx, c->ev_bare[1], 0);
+                        return;
+                    }
                     if (launch_cond_pairs(c->prec, q, (int)(bb - ba), c->sms, sx)) return;
                     // two lanes per row: the register-resident kernel where it exists
                     if (team == 2 && launch_cond_pair(q, (int)(bb - ba), sx)) return;
@@ -1088,6 +1112,7 @@ bmf_status run_batch(bmf_ctx *c, int sl0, int sl1, int n_sweeps, const bmf_draws
                 CUDA_TRY(c, cudaEventRecord(c->ev_cdone, c->st3));
                 CUDA_TRY(c, cudaStreamWaitEvent(c->st, c->ev_cdone, 0));
             }
+            CUDA_TRY(c, bare_err);
             if (keep && c->summary != BMF_SUMMARY_MM && r1 > r0)
                 CUDA_TRY(c, cudaMemcpyAsync(c->ring[f] + (kept - 1) * me.R * K + r0 * K, me.F + r0 * K,
                                             (size_t)(r1 - r0) * K * sizeof(double),
@@ -1629,10 +1654,11 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
         ok = ok && cudaStreamCreateWithPriority(&c->st3, cudaStreamNonBlocking, hi) == cudaSuccess;
         ok = ok && cudaStreamCreateWithPriority(&c->st4, cudaStreamNonBlocking, hi) == cudaSuccess;
         ok = ok && cudaStreamCreateWithPriority(&c->st5, cudaStreamNonBlocking, hi) == cudaSuccess;
+        ok = ok && cudaStreamCreateWithPriority(&c->st6, cudaStreamNonBlocking, hi) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess;
         for (cudaEvent_t *e : {&c->ev_fork, &c->ev_fac[0], &c->ev_fac[1], &c->ev_hyp[0], &c->ev_hyp[1],
                                &c->ev_cdone, &c->ev_tail, &c->ev_tail2, &c->ev_rmse, &c->ev_gen[0],
-                               &c->ev_gen[1]})
+                               &c->ev_gen[1], &c->ev_bare[0], &c->ev_bare[1]})
             ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
         for (cudaEvent_t &e : c->ev_copyq)
             ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
@@ -1692,10 +1718,23 @@ bmf_status bmf_init(bmf_ctx **out, const bmf_config *cfg, int64_t N, int64_t D, 
             ch[b].out = (int32_t)(sd.stat0 + (int64_t)b);
             ch[b].arena = f;
         }
+        std::vector<int32_t> bare;
+        sd.h_bare_ptr.assign(1, 0);
+        for (const CondBlock &b : sd.h_blocks) {
+            for (int64_t r = b.row0; r < b.row0 + b.n; ++r)
+                if (sd.h_obs[r] == sd.h_obs[r + 1]) bare.push_back((int32_t)r);
+            sd.h_bare_ptr.push_back((int64_t)bare.size());
+        }
+        if (c->prec != BMF_FP64 && K >= kPairsMinK && K <= kBareMaxK) {
+            sd.bare = c->mem.alloc<int32_t>(bare.size());
+            sd.bare_factor = c->mem.alloc<double>((K + ntri(K)) * bare.size());
+        }
         sd.blocks = c->mem.alloc<CondBlock>(sd.h_blocks.size());
         sd.chunks = c->mem.alloc<StatChunk>(ch.size());
         if (!c->mem.ok) return bail(BMF_E_OOM, "device allocation failed (block tables)");
         if (!ch.empty()) {
+            if (sd.bare && !bare.empty())
+                cudaMemcpy(sd.bare, bare.data(), bare.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
             cudaMemcpy(sd.blocks, sd.h_blocks.data(), ch.size() * sizeof(CondBlock), cudaMemcpyHostToDevice);
             cudaMemcpy(sd.chunks, ch.data(), ch.size() * sizeof(StatChunk), cudaMemcpyHostToDevice);
         }

@@ -530,13 +530,129 @@ __device__ __noinline__ void redo_rows(const CondParams &a, int64_t row0, unsign
     }
 }
 
+// Rows without observations whose prior is their own (K <= kBareMaxK): nothing but their prior and their
+// normals enters them, and no other row and no statistic waits for them.  x = L^{-T} (y + z) with
+// L L^T = Lambda_p and L y = b_p, which stay as they are while a call's sweeps draw z: FP64, the factor
+// once per call, the draws, K (K + 1) / 2 multiply-adds a row, beside the float pairs of the other rows.
+// 225,000 rows at K = 16, 62,000 of them such rows, us a half sweep: 541 with pairs for all, 1,240
+// with these drawn like redo_rows', 543 now.  (Above K = 16 redo_rows takes them: a thread's row no
+// longer fits in registers.)
+//
+// The factor, a thread per row, the matrix interleaved in shared memory (entry e of a row at e * 32), four
+// rows of a column at a time; out: [ntri(K) + K][n_all], entry by entry, 1 / L_jj on the diagonal (zero
+// in entry 0 of a row that is not positive definite), then y.
+__global__ void __launch_bounds__(32) bare_factor_kernel(const __grid_constant__ CondParams a, BareRows w)
+{
+    extern __shared__ double smd[];
+    constexpr int W = 32, BATCH = 16;   // loads of a row in flight
+    const int K = a.K, NT = ntri(K);
+    double *A = smd + threadIdx.x;      // the packed triangle, then the right-hand side as its row K
+    for (int64_t q = w.first + (int64_t)blockIdx.x * W + threadIdx.x; q < w.last; q += (int64_t)gridDim.x * W) {
+        const int64_t r = w.rows[q];
+        if (a.row_hslot[r] >= 0) continue;
+        for (int e0 = 0; e0 < NT + K; e0 += BATCH) {
+            double v[BATCH];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) {
+                const int e = min(e0 + u, NT + K - 1);
+                v[u] = e < NT ? a.prior_L[(int64_t)e * a.R + r] : a.prior_b[(int64_t)(e - NT) * a.R + r];
+            }
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u)
+                if (e0 + u < NT + K) A[(e0 + u) * W] = v[u];
+        }
+        bool ok = true;
+        for (int j = 0; j < K; ++j) {
+            double *Lj = A + tri(j, 0) * W;
+            double d = Lj[j * W];
+            for (int k = 0; k < j; ++k) d = fma(-Lj[k * W], Lj[k * W], d);
+            ok = ok && pivot_ok(d);
+            const double rs = ok ? rsqrt_full(d) : 0.0;
+            Lj[j * W] = rs;
+            for (int i0 = j + 1; i0 <= K; i0 += 4) {
+                double *Li[4], v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    Li[u] = A + tri(min(i0 + u, K), 0) * W;
+                    v[u] = Li[u][j * W];
+                }
+                for (int k = 0; k < j; ++k) {
+                    const double l = Lj[k * W];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = fma(-Li[u][k * W], l, v[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (i0 + u <= K) Li[u][j * W] = v[u] * rs;
+            }
+        }
+        if (!ok) {
+            atomicOr(&a.err->flags, ERR_NOT_PD);
+            atomicMin(&a.err->first_bad_row, (int)r);
+            A[0] = 0.0;
+        }
+        for (int e = 0; e < NT + K; ++e) w.factor[(int64_t)e * w.n_all + q] = A[e * W];
+    }
+}
+
+// The draws, a thread per row: a row's factor, normals and moment sums once through memory.
+template <int KM, typename GT>
+__global__ void __launch_bounds__(128) bare_draw_kernel(const __grid_constant__ CondParams a, BareRows w)
+{
+    const int K = a.K, NT = ntri(K);
+    const int64_t q = w.first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x, N = w.n_all;
+    if (q >= w.last) return;
+    const int64_t r = w.rows[q];
+    const double *F = w.factor + q;
+    if (a.row_hslot[r] >= 0 || F[0] == 0.0) return;
+    double x[KM];
+    const double *z = a.z + (r - a.row0) * K;
+#pragma unroll
+    for (int i = 0; i < KM; ++i) x[i] = i < K ? F[(int64_t)(NT + i) * N] + z[i] : 0.0;
+#pragma unroll
+    for (int i = KM - 1; i >= 0; --i)
+        if (i < K) {
+            double l[KM];
+#pragma unroll
+            for (int k = 0; k <= i; ++k) l[k] = F[(int64_t)tri(i, k) * N];
+            x[i] *= l[i];
+#pragma unroll
+            for (int k = 0; k < i; ++k) x[k] = fma(-l[k], x[i], x[k]);
+        }
+    GT *g = static_cast<GT *>(a.Xg) + r * a.ldg;
+#pragma unroll
+    for (int i = 0; i < KM; ++i)
+        if (i < K) {
+            a.X[r * K + i] = x[i];
+            g[i] = gathered<GT>(x[i], (float)x[i]);
+        }
+    for (int i = K; i < a.ldg; ++i) g[i] = gathered<GT>(0.0, 0.f);
+    if (!a.keep) return;
+    double s[KM];
+#pragma unroll
+    for (int i = 0; i < KM; ++i) s[i] = a.S1[(int64_t)min(i, K - 1) * a.R + r];
+#pragma unroll
+    for (int i = 0; i < KM; ++i)
+        if (i < K) a.S1[(int64_t)i * a.R + r] = s[i] + x[i];
+    if (!a.full) return;
+#pragma unroll
+    for (int i = 0; i < KM; ++i)
+        if (i < K) {
+            double *S = a.S2 + (int64_t)tri(i, 0) * a.R + r;
+#pragma unroll
+            for (int j = 0; j <= i; ++j) s[j] = S[(int64_t)j * a.R];
+#pragma unroll
+            for (int j = 0; j <= i; ++j) S[(int64_t)j * a.R] = fma(x[i], x[j], s[j]);
+        }
+}
+
 template <int T, int RMAX, typename GT>
 __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__ CondParams a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long redo_rest;   // rows of the block left for FP64
-    if (threadIdx.x == 0) redo_rest = 0ull;
-    __syncthreads();
+    __shared__ unsigned has[kCondBlock / 32];
+    __shared__ uint8_t order[kCondBlock];
     const int K = a.K, NT = ntri(K), KP = padded4(K);
     const int lane = threadIdx.x & 31, tl = threadIdx.x % T, tm = threadIdx.x / T;
     const int n_teams = blockDim.x / T;
@@ -545,16 +661,33 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
     double *xd = reinterpret_cast<double *>(Y + 2 * KP);   // z, then the state
     const CondBlock blk = a.blocks[blockIdx.x];
     const int64_t R = a.R;
+    // rows without observations are FP64's: the others are dealt to the block's parts and their teams
+    // without gaps (30,011 x 2,027 at K = 24, 20 sweeps: 14.8 -> 13.7 ms)
+    const int own = threadIdx.x;
+    const bool sums_of = own < blk.n && a.item_ptr[blk.row0 + own + 1] > a.item_ptr[blk.row0 + own];
+    if (own < kCondBlock) {
+        const unsigned v = __ballot_sync(0xffffffffu, sums_of);
+        if (lane == 0) has[own >> 5] = v;
+    }
+    __syncthreads();
+    const unsigned long long with = (unsigned long long)has[1] << 32 | has[0];
+    const int n_with = __popcll(with);
+    if (sums_of) order[__popcll(with & ((1ull << own) - 1ull))] = (uint8_t)own;
+    if (own == 0) {
+        const bool apart = a.bare_apart && a.row_hslot[blk.row0] < 0;
+        redo_rest = blockIdx.y > 0 || apart ? 0ull : ~with & (~0ull >> (kCondBlock - blk.n));
+    }
+    __syncthreads();
     const unsigned tmask = T == 32 ? 0xffffffffu : ((1u << T) - 1u) << (lane & ~(T - 1));
-    const int rows = kCondBlock / gridDim.y, q_end = min(blk.n, (int)(blockIdx.y + 1) * rows);
+    const int rows = kCondBlock / gridDim.y, q_end = min(n_with, (int)(blockIdx.y + 1) * rows);
     for (int q0 = blockIdx.y * rows; q0 < q_end; q0 += n_teams) {
-        const int q = q0 + tm;
-        const bool active = q < q_end;
-        const int64_t r = blk.row0 + (active ? q : 0);
+        const bool active = q0 + tm < q_end;
+        const int q = active ? order[q0 + tm] : 0;
+        const int64_t r = blk.row0 + q;
         bool bad = false, sums = false;
-        // G, r and the prior (teams past the block's rows carry an identity)
+        // G, r and the prior (teams without a row carry an identity)
         if (active) {
-            const int64_t i0 = a.item_ptr[r], i1 = a.item_ptr[r + 1];
+            const int64_t i0 = a.item_ptr[r];
             const int mi = a.multi_idx[r], h = a.row_hslot[r];
             const double tau_d = a.tau_row ? a.tau_row[r] : a.tau;
             const int64_t o0 = T == 4 ? a.obs_ptr[r] : 0, o1 = T == 4 ? a.obs_ptr[r + 1] : 0;
@@ -578,17 +711,12 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
                     }
             } else if (T == 4 && mi == kFusedRow) {
                 if constexpr (T == 4) team.own_gram(o0, (int)(o1 - o0));
-            } else if (i1 > i0) {
+            } else {
                 for (int i = tl; i < K; i += T) {
                     const float *src = pp + tri(i, 0);
                     fpair *dst = M + row_off(i);
                     for (int j = 0; j <= i; ++j) copy4(&dst[j].h, src + j);
                     copy4(&Y[i].h, pp + a.part_rhs + i);
-                }
-            } else {
-                for (int i = tl; i < K; i += T) {
-                    for (int j = 0; j <= i; ++j) M[row_off(i) + j].h = 0.f;
-                    Y[i].h = 0.f;
                 }
             }
             // prior + tau g, four entries at a time, the next four priors in flight
@@ -717,11 +845,37 @@ bool launch_cond_pairs(int prec, const CondParams &a, int n_blocks, int sms, cud
 {
     if (prec == BMF_FP64 || a.K < kPairsMinK || a.K > kPairsMaxK) return false;
     if (n_blocks <= 0) return true;
-    if (prec == BMF_FP32)
-        launch_pairs_t<float>(a, n_blocks, sms, st);
-    else
+    if (prec == BMF_BF16)
         launch_pairs_t<__nv_bfloat16>(a, n_blocks, sms, st);
+    else
+        launch_pairs_t<float>(a, n_blocks, sms, st);
     return true;
+}
+
+void launch_bare_factor(const CondParams &a, const BareRows &w, int sms, cudaStream_t st)
+{
+    const size_t smem = (size_t)32 * (ntri(a.K) + a.K) * sizeof(double);   // 39 KB at K = 16: five per SM
+    const int64_t blocks = std::min<int64_t>((int64_t)5 * sms, (w.last - w.first + 31) / 32);
+    if (blocks > 0) bare_factor_kernel<<<(int)blocks, 32, smem, st>>>(a, w);
+}
+
+template <typename GT>
+static void launch_draw_t(const CondParams &a, const BareRows &w, cudaStream_t st)
+{
+    const unsigned blocks = (unsigned)((w.last - w.first + 127) / 128);
+    if (a.K <= 12)
+        bare_draw_kernel<12, GT><<<blocks, 128, 0, st>>>(a, w);
+    else
+        bare_draw_kernel<kBareMaxK, GT><<<blocks, 128, 0, st>>>(a, w);
+}
+
+void launch_bare_draw(int prec, const CondParams &a, const BareRows &w, cudaStream_t st)
+{
+    if (w.last <= w.first) return;
+    if (prec == BMF_BF16)
+        launch_draw_t<__nv_bfloat16>(a, w, st);
+    else
+        launch_draw_t<float>(a, w, st);
 }
 
 }  // namespace bmf

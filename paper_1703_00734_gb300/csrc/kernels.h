@@ -88,6 +88,8 @@ struct CondParams {
     int *parts_done;             // [blocks], zero between launches: a conditional block's rows may be
                                  // split over several CUDA blocks (grid y), the last of which
                                  // forms the block's statistics
+    int bare_apart;              // float-pair draw: the launch leaves rows that have no observations
+                                 // and a prior of their own to launch_bare_draw
     DevError *err;
     // rows marked kFusedRow in multi_idx form their own Gram sums from their observations (in
     // list order), which the Gram pass skips: the row's list and the gathered partner copy
@@ -102,6 +104,16 @@ void launch_cond(int prec, const CondParams &a, int n_blocks, cudaStream_t st);
 // (cond_pairs.cu).  False for the others (nothing launched).
 constexpr int kPairsMinK = 9, kPairsMaxK = 48;
 bool launch_cond_pairs(int prec, const CondParams &a, int n_blocks, int sms, cudaStream_t st);
+// Beside it, at K <= kBareMaxK: the rows without observations [first, last) of a side's n_all, those that
+// have a prior of their own.  Their factors from their priors, then their draws.
+constexpr int kBareMaxK = 16;
+struct BareRows {
+    const int32_t *rows;
+    double *factor;              // [ntri(K) + K][n_all]
+    int64_t n_all, first, last;
+};
+void launch_bare_factor(const CondParams &a, const BareRows &w, int sms, cudaStream_t st);
+void launch_bare_draw(int prec, const CondParams &a, const BareRows &w, cudaStream_t st);
 // multi_idx of a row whose Gram sums the conditional draw forms itself: 13 <= K <= 16 (the
 // two-lane and team conditionals) and 1 to kFuseMaxObs observations in one work item.  Such a
 // row's partner rows are few and mostly cached, where its Gram partials would be a round trip
