@@ -127,8 +127,10 @@ typedef enum {
 /* Precision of the gathered factor copies and of the Gram accumulation.  The
  * hyperparameter step, moments and states are FP64 in all modes, and so are the conditional
  * assembly, Cholesky, solves and draws, except that the reduced-precision modes take them in pairs
- * of floats (48 bits, twice what their Gram sums carry) at 9 <= K <= 48, with FP64 for rows whose
- * range or conditioning needs it.
+ * of floats at 9 <= K <= 48.  An operation in pairs is off by at most 2^-44, and a pivot may lose
+ * 20 bits to cancellation, which leaves it the 2^-24 of the FP32 sums it is formed from.  FP64 draws
+ * the rows whose sums make up less than 2^-16 of every diagonal entry of their precision (above all
+ * rows without observations) and those whose range or conditioning pairs cannot hold.
  * FP32 gathers at K > 16 reach the tensor cores as split TF32 (three products per tile, close to
  * FP32 products); BMF_TF32 keeps FP32 gathers but takes one TF32 product per tile (operands
  * rounded to 10-bit mantissas) at K > 16, and is BMF_FP32 at K <= 16. */

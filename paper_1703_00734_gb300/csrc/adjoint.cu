@@ -431,7 +431,7 @@ void launch_adjoint(const AdjointParams &a, int grid, cudaStream_t st)
 }
 
 // Langevin move on the FP32 factors X and W: out = theta + (eps/2) grad + sqrt(eps) xi (out may be
-// theta itself; padding kept as it is, zero in a copy).
+// theta itself; padding is kept, and copied where out is not theta).
 __global__ void langevin_kernel(const float *X, const float *W, const float *gX, const float *gW, float *oX,
                                 float *oW, const float *xi, int64_t n_x, int64_t n_w, int K, int ld, float eps)
 {

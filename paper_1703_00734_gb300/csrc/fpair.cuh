@@ -1,6 +1,6 @@
 // fpair.cuh -- arithmetic on float pairs: a value is the unevaluated sum h + l of two floats with
-// |l| <= ulp(h) / 2, about 48 significant bits (Dekker 1971, Knuth's two-sum; with FMA the error
-// of a product is one instruction).
+// |l| <= ulp(h) / 2 (below ulp(h) from split(), which truncates), about 48 significant bits (Dekker
+// 1971, Knuth's two-sum; with FMA the error of a product is one instruction).
 //
 // Why: on this GPU the FP64 pipe takes a warp instruction every 17 clocks per SM and the FP32
 // pipes four every clock.  A multiply-add of pairs is 12 FP32 instructions (3.3 clocks), so the
@@ -116,7 +116,9 @@ __device__ __forceinline__ bool pair_diag(float h) { return h >= 0x1p-60f && h <
 
 // The top 24 bits of x and the following 24 as a pair, on the integer pipe (the conversion
 // instructions between FP32 and FP64 run on the FP64 pipe): relative error below 2^-48 down to
-// 2^-78; x below 2^-126 reads as zero.  x must pass pair_below.
+// 2^-78; x below 2^-126 reads as zero.  Not normalised: h is truncated, so l has its sign and may be
+// just below ulp(h); what takes it as a factor loses at most one of the 48 bits.  x must pass
+// pair_below.
 __device__ __forceinline__ fpair split(double x)
 {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);

@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(256) hyper_kernel(HyperParams a)
     __syncthreads();
     if (flag) goto fail;
     if constexpr (FAST) {
-        if (t < 32) {   // column by column, lane l holding v_l (K <= 32)
+        if (t < 32) {   // column by column, lane l holding v_l (K <= kHyperFastMaxK)
             double v0 = t < K ? v[t] : 0.0;
             for (int i = K - 1; i >= 0; --i) {
                 const double x = __shfl_sync(0xffffffffu, v0, i) * rinv[i];
