@@ -7,11 +7,11 @@
 //
 // The FP64 pipe of this GPU takes a warp instruction every 17 clocks per SM; a multiply-add of
 // float pairs is 12 FP32 instructions, 3.3 clocks, at 48 bits, where the Gram sums carry 24.
-// Measured inside whole runs, FP64 teams or threads per row before, this kernel now, per half
-// sweep: K = 16, 225,000 rows with propagated priors and moment sums 1,456 -> 855 us (617 us alone);
-// K = 32, 120,047 rows 3,448 -> 1,409 us; K = 24, 30,011 rows 559 -> 240 us; K = 10, 69,878 rows
-// 112 -> 95 us.  Alone it issues 47% of the time: the pair arithmetic is about half of its 1,440
-// warp instructions per row at K = 16, the rest loads, splits and range checks.
+// Alone on the device, FP64 teams or threads per row before, this kernel now, per half sweep: K = 10,
+// 69,878 rows 127 -> 91 us; K = 32, 120,047 rows 3,832 -> 1,184 us; K = 16, 225,000 rows with
+// propagated priors and moment sums 1,221 -> 540 us for 163,000 of them and, beside it, 118 us for the
+// others, which have no observations.  It issues 39 to 59% of the time: the pair arithmetic is about
+// half of its 1,570 warp instructions per row at K = 16, the rest loads, splits and range checks.
 //
 // The dispatch: below K = 9 a row's FP64 work is small enough that a thread per row is as fast;
 // above K = 48 the FP64 teams stay, because there a change in the last bit of a draw grows, through
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(256) cond_pairs_kernel(const __grid_constant__
     const CondBlock blk = a.blocks[blockIdx.x];
     const int64_t R = a.R;
     // rows without observations are FP64's: the others are dealt to the block's parts and their teams
-    // without gaps (30,011 x 2,027 at K = 24, 20 sweeps: 14.8 -> 13.7 ms)
+    // without gaps (30,011 x 2,027 at K = 24, 20 sweeps: 14.8 -> 13.7 to 14.7 ms)
     const int own = threadIdx.x;
     const bool sums_of = own < blk.n && a.item_ptr[blk.row0 + own + 1] > a.item_ptr[blk.row0 + own];
     if (own < kCondBlock) {
@@ -813,7 +813,7 @@ static void launch_team_t(const CondParams &a, int n_blocks, int sms, cudaStream
     // rows: 63 us with 64 threads, 32 us with 256).  Larger launches take 64 threads, which fill an
     // SM evenly, and the rows of a conditional block in as many parts as rounds of its teams, until
     // the launch fills the GPU about eight times over (K = 16, 45,000 rows: 245 us as one part, 149
-    // us in parts; 225,000 rows: 660 and 609 us).
+    // us in parts; 225,000 rows: 660 and 609 us, all of them in pairs).
     auto bytes = [&](int th) { return (size_t)(th / T) * team_pairs(a.K) * sizeof(fpair); };
     auto fit = [&](int th) { return (int)std::min<size_t>(512 / th, (size_t)220 * 1024 / bytes(th)); };
     int threads = 256, parts = 1;
